@@ -196,7 +196,6 @@ NCU_TRAFFIC = {
     "spec_prod32_kernel": (1923.2, "f34fb6e78487019a", "atom-frequency of one type"),
     "spec_adj32_kernel": (7533.4, "8e9f1b2f0231170c", "atom-frequency of one type"),
     "spec_pi32_kernel": (2121.4, "3f8eabc933beac4b", "type-atom-frequency"),
-    "spec_gradg32_kernel": (1863.7, "aa646c7c1d04f57d", "atom-frequency of one type"),
     "spec_prod_tc_kernel": (1865.6, "b6487e717de45e49", "atom-frequency of one type"),
 }
 

@@ -2,7 +2,7 @@
 // FP64_FFT) and FP32 (spec_prod32_kernel, mode FP32_FFT), the symmetrisation, the workspace layout and the
 // drivers (device buffers, and the pipelined variant behind the host-buffer entry point). Mode F16X3_FFT runs the
 // same FP32 transforms with the block products of sse_spectral_tc.cu on the tensor cores.
-#include "sse_spectral.cuh"
+#include "sse_prod32.cuh"
 
 namespace sse {
 namespace {
@@ -127,187 +127,6 @@ __global__ void spec_prod_kernel(ProdCfg c, sse_dims d, FreqMap fm, const int32_
     }
 }
 
-// ---------------------------------------------------------------------------
-// phonon self-energy, Eq. (4): per (a, slot s, frequency)
-//   C^_ij(kappa,eps) = tr( dH_i^H G^t_a(kappa,eps) dH_j G^t'_b(-kappa,-eps) ),
-// the transform of the correlation sum_{k,E} tr(dH_i^H G^t_a(E+l, k+q) dH_j G^t'_b(E, k)) over the lags
-// (q, l); slot NB (the diagonal block) is the sum over the bonds.
-// ---------------------------------------------------------------------------
-// FP32 block products with register tiles. The FP32 pipe issues 64x the FP64 rate, so the scalar
-// kernel above becomes bound by shared-memory bandwidth (two scalar loads per FMA). Here each
-// thread computes a 2 x 2 tile of the (zero-padded, Np = Norb rounded up to even) block for one
-// frequency, with G^ and dH stored transposed so that every operand pair is one 8-byte load:
-// per reduction step 12 FMA for 6 loads. Same arithmetic as spec_prod_kernel (Gauss MACs).
-// ---------------------------------------------------------------------------
-struct Prod32Cfg {
-    int Np, TN, T, F, threads, fchunk;
-    int pl;      // floats per Np x Np plane
-    int gs, us;  // floats per frequency of the G^ and U regions, padded to 16 mod 32 (see below)
-    int off_A, off_G, off_K, off_U, smem;
-};
-
-
-// FP32 products use the 4-multiply complex MAC on (re, im) planes: with shared-memory bandwidth, not the FP32
-// pipe, the limit, two planes per operand (4 loads per 16 FMAs of a 2 x 2 tile) beat the 3-multiply form's
-// three planes (6 loads per 12 FMAs). U_i = G^ W_i is formed as sum_j K_ij P_j with P_j = G^ A_j^H, so the
-// weight blocks W_i never pass through shared memory.
-Prod32Cfg make_prod32_cfg(const sse_dims& d, size_t nfreq) {
-    Prod32Cfg c{};
-    c.Np = d.Norb + (d.Norb & 1);
-    c.TN = c.Np / 2;
-    c.T = c.TN * c.TN;
-    c.pl = c.Np * c.Np;
-    const int pb = c.pl * 4;  // bytes per plane
-    auto a16 = [](int x) { return (x + 15) & ~15; };
-    c.gs = bank_pad16(2 * c.pl);
-    c.us = bank_pad16(6 * c.pl);
-    c.F = pick_frequencies(c.T, [&](int F) { return (long)d.NB * 6 * pb + F * (4L * (c.gs + c.us) + 9 * 8) + 64; });
-    c.threads = ((c.F * c.T + 31) / 32) * 32;
-    c.off_A = 0;                                  // [NB][3 dir][2 planes] dH transposed: AT[l][m] = dH[m][l]
-    c.off_G = a16(c.off_A + d.NB * 6 * pb);       // [F][gs] G^ transposed (2 planes): GT[l][m] = G^[m][l]
-    c.off_K = a16(c.off_G + c.F * c.gs * 4);      // [F][9] float2
-    c.off_U = a16(c.off_K + c.F * 9 * 8);         // [F][us] U_i row-major (3 i x 2 planes)
-    c.smem = a16(c.off_U + c.F * c.us * 4);
-    const size_t nA = (size_t)(d.a_end - d.a_begin);
-    size_t want = (size_t)152 * 2 * 8;
-    size_t chunks = (want + nA - 1) / (nA ? nA : 1);
-    if (chunks < 1) chunks = 1;
-    size_t fc = (nfreq + chunks - 1) / chunks;
-    fc = ((fc + c.F - 1) / c.F) * c.F;
-    c.fchunk = (int)(fc < 1 ? 1 : fc);
-    return c;
-}
-
-__global__ void spec_prod32_kernel(Prod32Cfg c, sse_dims d, FreqMap fm, const int32_t* __restrict__ nbr,
-                                   const double2* __restrict__ dH, const float2* __restrict__ Ghat,
-                                   const float2* __restrict__ Khat, float2* __restrict__ Shat, double scale,
-                                   unsigned* __restrict__ status) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int Norb = d.Norb, Np = c.Np, pl = c.pl, nel = Norb * Norb;
-    const int la = blockIdx.x;
-    const int a = d.a_begin + la;
-    const size_t nA = (size_t)(d.a_end - d.a_begin);
-    const size_t i_begin = (size_t)blockIdx.y * c.fchunk;
-    const size_t i_end = min(fm.count, i_begin + c.fchunk);
-    float* sA = reinterpret_cast<float*>(smem + c.off_A);
-    float* sG = reinterpret_cast<float*>(smem + c.off_G);
-    float2* sK = reinterpret_cast<float2*>(smem + c.off_K);
-    float* sU = reinterpret_cast<float*>(smem + c.off_U);
-    const int tid = threadIdx.x;
-    const int fl = tid / c.T, tt = tid - fl * c.T;
-    const int m0 = 2 * (tt / c.TN), n0 = 2 * (tt % c.TN);
-    const bool lane = fl < c.F;
-
-    // dH planes, transposed and zero-padded: AT[s][dir][plane][l][m] = dH(a,s,dir)[m][l]
-    for (int i = tid; i < d.NB * 3 * pl; i += blockDim.x) {
-        const int sd = i / pl, e = i - sd * pl;
-        const int l = e / Np, m = e - l * Np;
-        double2 v = make_double2(0.0, 0.0);
-        if (l < Norb && m < Norb) v = dH[((size_t)a * d.NB * 3 + sd) * nel + m * Norb + l];
-        float* P = sA + (size_t)sd * 2 * pl;
-        P[e] = (float)v.x;
-        P[pl + e] = (float)v.y;
-    }
-    for (int s = 0; s < d.NB; ++s) {
-        const int b = nbr[(size_t)a * d.NB + s];
-        if ((b < 0 || b >= d.NA) && tid == 0) atomicOr(status, DEV_BAD_NEIGHBOUR);
-    }
-    __syncthreads();
-
-    for (size_t i0 = i_begin; i0 < i_end; i0 += c.F) {
-        const bool act = lane && i0 + fl < i_end;
-        const size_t f = act ? freq_of(fm, i0 + fl) : 0;
-        float accr[4] = {0, 0, 0, 0}, acci[4] = {0, 0, 0, 0};  // the 2 x 2 tile of sum_s sum_i dH_i U_i
-        for (int s = 0; s < d.NB; ++s) {
-            const int b = nbr[(size_t)a * d.NB + s];
-            const bool bok = b >= 0 && b < d.NA;
-            // G^_b(f) -> GT planes: element (m, n) goes to GT[n][m]
-            if (lane) {
-                float* Gp = sG + (size_t)fl * c.gs;
-#pragma unroll
-                for (int dm = 0; dm < 2; ++dm)
-#pragma unroll
-                    for (int dn = 0; dn < 2; ++dn) {
-                        const int m = m0 + dm, n = n0 + dn;
-                        float2 g = make_float2(0.f, 0.f);
-                        if (act && bok && m < Norb && n < Norb) g = Ghat[(f * d.NA + b) * nel + m * Norb + n];
-                        const int o = n * Np + m;
-                        Gp[o] = g.x;
-                        Gp[pl + o] = g.y;
-                    }
-            }
-            for (int i = tid; i < c.F * 9; i += blockDim.x) {
-                const int fk = i / 9, ij = i - fk * 9;
-                float2 k = make_float2(0.f, 0.f);
-                if (i0 + fk < i_end && bok) k = Khat[((freq_of(fm, i0 + fk) * nA + la) * d.NB + s) * 9 + ij];
-                sK[i] = k;
-            }
-            __syncthreads();
-            const float* A = sA + (size_t)s * 6 * pl;
-            // P_j = G^ A_j^H for the three j at once: P_j[m][n] = sum_l GT[l][m] conj(AT_j[l][n]);
-            // U_i = G^ W_i = sum_j K_ij P_j
-            if (lane) {
-                const float* Gp = sG + (size_t)fl * c.gs;
-                float pr[3][4] = {}, pim[3][4] = {};
-                for (int l = 0; l < Norb; ++l) {
-                    const float2 gr = ld2(Gp + l * Np + m0), gi = ld2(Gp + pl + l * Np + m0);
-#pragma unroll
-                    for (int j = 0; j < 3; ++j)
-                        cmac2x2<false, true>(pr[j], pim[j], gr, gi, ld2(A + (size_t)j * 2 * pl + l * Np + n0),
-                                             ld2(A + (size_t)j * 2 * pl + pl + l * Np + n0));
-                }
-                const float2* K = sK + fl * 9;
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    float ur[4] = {0, 0, 0, 0}, ui[4] = {0, 0, 0, 0};
-#pragma unroll
-                    for (int j = 0; j < 3; ++j) {
-                        const float2 k = K[i * 3 + j];
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            ur[q] = fmaf(k.x, pr[j][q], ur[q]);
-                            ur[q] = fmaf(-k.y, pim[j][q], ur[q]);
-                            ui[q] = fmaf(k.x, pim[j][q], ui[q]);
-                            ui[q] = fmaf(k.y, pr[j][q], ui[q]);
-                        }
-                    }
-                    float* Up = sU + (size_t)fl * c.us + (size_t)i * 2 * pl;
-#pragma unroll
-                    for (int dm = 0; dm < 2; ++dm) {
-                        float* o = Up + (m0 + dm) * Np + n0;
-                        st2(o, ur[dm * 2], ur[dm * 2 + 1]);
-                        st2(o + pl, ui[dm * 2], ui[dm * 2 + 1]);
-                    }
-                }
-            }
-            __syncthreads();
-            // acc += sum_i dH_i U_i: acc[m][n] += sum_l AT_i[l][m] U_i[l][n]
-            if (lane) {
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    const float* Ap = A + (size_t)i * 2 * pl;
-                    const float* Up = sU + (size_t)fl * c.us + (size_t)i * 2 * pl;
-                    for (int l = 0; l < Norb; ++l) {
-                        const float2 ar = ld2(Ap + l * Np + m0), ai = ld2(Ap + pl + l * Np + m0);
-                        const float2 vr = ld2(Up + l * Np + n0), vi = ld2(Up + pl + l * Np + n0);
-                        cmac2x2<false, false>(accr, acci, ar, ai, vr, vi);
-                    }
-                }
-            }
-            __syncthreads();  // sG, sK, sU are rewritten for the next bond
-        }
-        if (act) {
-            const float sc = (float)scale;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int m = m0 + q / 2, n = n0 + (q & 1);
-                if (m < Norb && n < Norb)  // i*scale*(re + i im)
-                    Shat[(f * nA + la) * nel + m * Norb + n] = make_float2(-sc * acci[q], sc * accr[q]);
-            }
-        }
-    }
-}
-
 // (S - S^H)/2 on the blocks of atoms in range
 __global__ void symmetrize_kernel(sse_dims d, double2* __restrict__ S) {
     const int Norb = d.Norb, nel = Norb * Norb;
@@ -362,8 +181,10 @@ bool spectral_supported(const sse_dims& d) {
            make_prod_cfg(d, (size_t)d.Nkz * L).smem <= 227 * 1024;
 }
 
+// The FP32 product kernel takes every block size and bond count of spectral_supported.
 bool spectral_fwd_supported(const sse_dims& d, bool fp32) {
-    return spectral_supported(d) && (!fp32 || make_prod32_cfg(d, 1).smem <= 227 * 1024);
+    (void)fp32;
+    return spectral_supported(d);
 }
 
 size_t spectral_fwd_workspace(const sse_dims& d) { return spec_layout(d).total; }
@@ -416,12 +237,11 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
         }
     }
     const ProdCfg pc = make_prod_cfg(d, fm.count, (int)sizeof(T));
-    const Prod32Cfg pc32 = make_prod32_cfg(d, fm.count);
-    const bool tiled = sizeof(T) == 4;  // FP32: register-tiled kernel
-    if ((e = tiled ? cudaFuncSetAttribute(spec_prod32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pc32.smem)
-                   : cudaFuncSetAttribute(spec_prod_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          pc.smem)) != cudaSuccess)
-        return e;
+    constexpr bool tiled = sizeof(T) == 4;  // FP32: register-tiled kernel
+    if constexpr (!tiled)
+        if ((e = cudaFuncSetAttribute(spec_prod_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, pc.smem)) !=
+            cudaSuccess)
+            return e;
     double2* S[2] = {S_less, S_greater};
     if (pipe && (e = cudaStreamWaitEvent(st, pipe->inputs, 0)) != cudaSuccess) return e;
     for (int t = 0; t < 2; ++t) {
@@ -450,12 +270,9 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
                                  reinterpret_cast<const float2*>(Kh), reinterpret_cast<float2*>(Sh), p.scale, status,
                                  st);
             if (e != cudaSuccess) return e;
-        } else if (tiled) {
-            const size_t gy = (fm.count + pc32.fchunk - 1) / pc32.fchunk;
-            SSE_TIMED("spec_prod32_kernel", st,
-                      spec_prod32_kernel<<<dim3((unsigned)nA, (unsigned)gy), pc32.threads, pc32.smem, st>>>(
-                          pc32, d, fm, p.nbr, p.dH, reinterpret_cast<const float2*>(Gh),
-                          reinterpret_cast<const float2*>(Kh), reinterpret_cast<float2*>(Sh), p.scale, status));
+        } else if constexpr (tiled) {
+            e = launch_prod32<false>(TileArgs{d, fm, p.nbr, nullptr, nullptr, p.dH, Gh, Kh, Sh, p.scale, status}, nA, st);
+            if (e != cudaSuccess) return e;
         } else {
             const size_t gy = (fm.count + pc.fchunk - 1) / pc.fchunk;
             SSE_TIMED("spec_prod_kernel", st,
