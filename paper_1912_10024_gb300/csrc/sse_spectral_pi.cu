@@ -1,6 +1,6 @@
 // Pi of Eq. (4) through the transforms: the per-frequency half products and traces in FP64 (spec_pi_kernel) and
 // FP32 (spec_pi32_kernel), the store of the inverse transform, the 3x3 symmetrisation and the driver.
-#include "sse_spectral.cuh"
+#include "sse_prod32.cuh"
 
 namespace sse {
 namespace {
@@ -169,218 +169,281 @@ spec_pi_kernel(PiCfg c, sse_dims d, FreqMap fm, const int32_t* __restrict__ nbr,
 }
 
 // ---------------------------------------------------------------------------
-// FP32 phonon self-energy (mode FP32_FFT): the half products P_i = dH_i^H X^ and R_j = dH_j Y^ three at a time
-// on 2 x 2 register tiles (4-multiply MACs on (re, im) planes); R_j goes to shared memory transposed, so each
-// thread forms its tile's part of tr(P_i R_j) from P_i in registers; the parts are summed over the tile threads
-// in a fixed order.
+// FP32 phonon self-energy (mode FP32_FFT). A thread owns the 2 x 2 pairs (m, n) of P_i[m][n] (P_i = dH_i^H X^) and of
+// R_j[n][m] (R_j = dH_j Y^) for the three i and j and for NF frequencies, so its part of every trace
+// tr(P_i R_j) = sum_mn P_i[m][n] R_j[n][m] is formed from its own registers; the parts are summed over the tile's
+// threads in a fixed order.
+//
+// What bounds it: the FP32 pipe and the shared-memory return path (128 bytes per clock and SM; see sse_prod32.cuh). The
+// coupling blocks are the same for every frequency, so NF frequencies per thread raise the FMAs per float loaded from 3
+// (one frequency, with R_j exchanged through shared memory) to 4.8 (NF = 2) and 6 (NF = 3). FMAs are issued in
+// pairs: over m for P, over n for R, with X^ and Y^ duplicated. FinFET workload: 55.1 -> 38.7 ms for Pi^< and Pi^>
+// (0.58 of the FP32 pipe); NF = 2 with three CTAs per SM (168 registers) is taken since it measured 38.7 ms against
+// 42.0 for NF = 2 with two CTAs and 40.7 for NF = 3 with two: warps to cover the latencies count for more than loads.
 // ---------------------------------------------------------------------------
-constexpr int kPi32MaxThreads = 256;  // <= 128 registers at two CTAs per SM
-
-struct Pi32Cfg {
-    int Np, TN, T, pl, F, threads, fchunk;
-    int xs, rs;  // floats per frequency of the X^ / Y^ regions and the R_j region, bank-padded
-    int off_A, off_X, off_Y, off_R, off_self, smem;
+template <int NP>
+struct PiShape {
+    static constexpr int TN = NP / 2, T = TN * TN;  // pairs per block edge, threads per frequency set
+    static constexpr int TP = T | 1;                // trace parts per (frequency, ij): an odd stride spreads the banks
+    static constexpr int NF = 2;                    // frequencies per thread (see above)
+    static constexpr int FG = 128 / T;              // frequency sets per CTA
+    static constexpr int F = FG * NF;
+    static constexpr int THREADS = (FG * T + 31) / 32 * 32;
+    static constexpr int CTAS = 3;
+    // floats of X^ or Y^ per frequency: two sets in one warp start 2 NP banks apart, so their rows do not collide
+    // (blocks of up to 4 x 4: no padding, the copies would be mostly padding)
+    static constexpr int XS = NP * NP * 2 + (NP <= 4 ? 0 : ((2 * NP - NP * NP * 2) % 32 + 32) % 32);
+    static constexpr int AB = 3 * NP * TN * 4;      // floats of one bond's dH in one of its two layouts
 };
 
-Pi32Cfg make_pi32_cfg(const sse_dims& d, size_t nfreq) {
-    Pi32Cfg c{};
-    c.Np = d.Norb + (d.Norb & 1);
-    c.TN = c.Np / 2;
-    c.T = c.TN * c.TN;
-    c.pl = c.Np * c.Np;
-    const int pb = c.pl * 4;
+struct PiTileCfg {
+    int fchunk, nchunks, nres;
+    int off_X, off_Y, off_P, off_self, off_F, smem;
+};
+
+template <int NP>
+PiTileCfg make_pi_tile_cfg(const sse_dims& d, size_t nfreq) {
+    using S = PiShape<NP>;
     auto a16 = [](int x) { return (x + 15) & ~15; };
-    // per CTA: every bond's dH row-major and transposed (12 planes per bond); per frequency X^, Y^ (4 planes),
-    // R_j transposed (6 planes; the trace parts reuse them) and the diagonal-block sums (9 float2)
-    c.xs = bank_pad16(2 * c.pl);
-    c.rs = bank_pad16(6 * c.pl);
-    c.F = pick_frequencies(
-        c.T, [&](int F) { return (long)d.NB * 12 * pb + F * (4L * (2 * c.xs + c.rs) + 9 * 8) + 96; }, 128,
-        kPi32MaxThreads);
-    c.threads = ((c.F * c.T + 31) / 32) * 32;
-    c.off_A = 0;                               // [NB][3][4 planes: re, im row-major; re, im transposed]
-    c.off_X = a16(c.off_A + d.NB * 12 * pb);     // [F][xs] X^ row-major (2 planes)
-    c.off_Y = a16(c.off_X + c.F * c.xs * 4);     // [F][xs] Y^ row-major
-    c.off_R = a16(c.off_Y + c.F * c.xs * 4);     // [F][rs] R_j transposed (3 j x 2 planes)
-    c.off_self = a16(c.off_R + c.F * c.rs * 4);  // [F][9] float2
-    c.smem = a16(c.off_self + c.F * 9 * 8);
+    PiTileCfg c{};
+    auto place = [&](int nres) {
+        c.nres = nres;
+        c.off_X = nres * 2 * S::AB * 4;
+        c.off_Y = c.off_X + S::F * S::XS * 4;
+        c.off_P = c.off_Y + S::F * S::XS * 4;
+        c.off_self = a16(c.off_P + S::F * 9 * S::TP * 8);
+        c.off_F = c.off_self + S::F * 9 * 8;
+        c.smem = a16(c.off_F + 4 * S::F * 4);
+        return c.smem;
+    };
+    // every bond's dH stays resident where it fits beside the buffers of CTAS CTAs
+    if (place(d.NB) > (227 / S::CTAS - 1) * 1024) place(1);
+    // tiles per CTA: enough CTAs for ~8 waves, at most 8 tiles (dH is staged per CTA)
     const size_t nA = (size_t)(d.a_end - d.a_begin);
-    size_t want = (size_t)152 * 2 * 8;
-    size_t chunks = (want + 2 * nA - 1) / (nA ? 2 * nA : 1);
-    if (chunks < 1) chunks = 1;
-    size_t fc = (nfreq + chunks - 1) / chunks;
-    fc = ((fc + c.F - 1) / c.F) * c.F;
-    c.fchunk = (int)(fc < 1 ? 1 : fc);
+    const size_t tiles = (nfreq + S::F - 1) / S::F;
+    size_t per = tiles * 2 * nA / ((size_t)152 * S::CTAS * 8);
+    per = per < 1 ? 1 : per > 8 ? 8 : per;
+    c.fchunk = (int)per;
+    c.nchunks = (int)((tiles + per - 1) / per);
     return c;
 }
 
-__global__ void __launch_bounds__(kPi32MaxThreads, 2)
-spec_pi32_kernel(Pi32Cfg c, sse_dims d, FreqMap fm, const int32_t* __restrict__ nbr, const double2* __restrict__ dH,
+template <int NP, int ODD>
+__global__ void __launch_bounds__(PiShape<NP>::THREADS, PiShape<NP>::CTAS)
+spec_pi32_kernel(PiTileCfg c, sse_dims d, FreqMap fm, const int32_t* __restrict__ nbr, const double2* __restrict__ dH,
                  const float2* __restrict__ Gl_hat, const float2* __restrict__ Gg_hat, float2* __restrict__ Cl_hat,
                  float2* __restrict__ Cg_hat, unsigned* __restrict__ status) {
+    using S = PiShape<NP>;
+    using Cp = TileCopy<NP, ODD>;
+    constexpr int N = NP - ODD, nel = N * N, NF = S::NF, F = S::F, XS = S::XS, nt = S::THREADS;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int Norb = d.Norb, Np = c.Np, pl = c.pl, nel = Norb * Norb, T = c.T;
-    const int la = blockIdx.x;
-    const int a = d.a_begin + la;
-    const int t = blockIdx.z;
+    // [res][P: [3 i][NP l][TN m] (re, re, im, im) of dH_i[l][m]; R: [3 j][NP l][TN n] of dH_j[n][l]]
+    float* sA = reinterpret_cast<float*>(smem);
+    float* sX = reinterpret_cast<float*>(smem + c.off_X);  // [F][NP l][NP n]
+    float* sY = reinterpret_cast<float*>(smem + c.off_Y);  // [F][NP l][NP m]
+    float2* sP = reinterpret_cast<float2*>(smem + c.off_P);      // [F][9][TP] trace parts
+    float2* sSelf = reinterpret_cast<float2*>(smem + c.off_self);  // [F][9] diagonal-block sums
+    int* sF = reinterpret_cast<int*>(smem + c.off_F);            // [2 tiles][f, -f][F], -1: none
+    const int tid = threadIdx.x, la = blockIdx.x, a = d.a_begin + la, t = blockIdx.z, slots = d.NB + 1;
     const float2* X_hat = t == 0 ? Gl_hat : Gg_hat;  // G^t of atom a
     const float2* Y_hat = t == 0 ? Gg_hat : Gl_hat;  // G^t' of the neighbour
     float2* C_hat = t == 0 ? Cl_hat : Cg_hat;
     const size_t nA = (size_t)(d.a_end - d.a_begin);
-    const size_t i_begin = (size_t)blockIdx.y * c.fchunk;
-    const size_t i_end = min(fm.count, i_begin + c.fchunk);
-    float* sA = reinterpret_cast<float*>(smem + c.off_A);
-    float* sX = reinterpret_cast<float*>(smem + c.off_X);
-    float* sY = reinterpret_cast<float*>(smem + c.off_Y);
-    float* sR = reinterpret_cast<float*>(smem + c.off_R);
-    float2* sSelf = reinterpret_cast<float2*>(smem + c.off_self);
-    const int tid = threadIdx.x;
-    const int fl = tid / T, tt = tid - fl * T;
-    const int m0 = 2 * (tt / c.TN), n0 = 2 * (tt % c.TN);
-    const bool lane = fl < c.F;
-    const int slots = d.NB + 1;
+    const int ntiles = (int)((fm.count + F - 1) / F);
+    const int tile0 = blockIdx.y * c.fchunk, tile1 = min(ntiles, tile0 + c.fchunk);
+    const bool resident = c.nres >= d.NB;
+    const int fs = tid / S::T, tt = tid - fs * S::T;
+    const int mp = tt / S::TN, np = tt - mp * S::TN;
+    const bool lane = fs < S::FG;
 
-    // dH planes of every bond, zero-padded: row-major A[l][n] and transposed AT[l][m] = A[m][l]
-    for (int i = tid; i < d.NB * 3 * pl; i += blockDim.x) {
-        const int si = i / pl, e = i - si * pl;
-        const int r = e / Np, q = e - r * Np;
-        double2 v = make_double2(0.0, 0.0), w = make_double2(0.0, 0.0);
-        if (r < Norb && q < Norb) {
-            v = dH[((size_t)a * d.NB * 3 + si) * nel + r * Norb + q];
-            w = dH[((size_t)a * d.NB * 3 + si) * nel + q * Norb + r];
+    auto stage_A = [&](int s, int slot) {
+        const double2* H = dH + ((size_t)a * d.NB + s) * 3 * nel;
+        float* P = sA + (size_t)slot * 2 * S::AB;
+        float* R = P + S::AB;
+        for (int i = tid; i < 3 * NP * NP; i += nt) {
+            const int j = i / (NP * NP), e = i - j * (NP * NP), r = e / NP, q = e - r * NP;
+            float2 v = make_float2(0.f, 0.f);  // dH_j[r][q]
+            if (r < N && q < N) {
+                const double2 h = H[j * nel + r * N + q];
+                v = make_float2((float)h.x, (float)h.y);
+            }
+            float* o = P + ((j * NP + r) * S::TN + q / 2) * 4 + (q & 1);
+            o[0] = v.x;
+            o[2] = v.y;
+            o = R + ((j * NP + q) * S::TN + r / 2) * 4 + (r & 1);
+            o[0] = v.x;
+            o[2] = v.y;
         }
-        float* P = sA + (size_t)si * 4 * pl;
-        P[e] = (float)v.x;
-        P[pl + e] = (float)v.y;
-        P[2 * pl + e] = (float)w.x;
-        P[3 * pl + e] = (float)w.y;
-    }
+    };
+    auto freq_table = [&](int tile) {
+        int* f = sF + (tile & 1) * 2 * F;
+        for (int i = tid; i < F; i += nt) {
+            const size_t ix = (size_t)tile * F + i;
+            const bool ok = ix < fm.count;
+            const size_t g = ok ? freq_of(fm, ix) : 0;
+            f[i] = ok ? (int)g : -1;
+            f[F + i] = ok ? (int)freq_neg(fm, g) : -1;
+        }
+    };
+    auto issue_one = [&](float* dst, const int* fq, const float2* src, int atom, bool aok) {
+        for (int i = tid; i < F * Cp::ITEMS; i += nt) {
+            const int f = i / Cp::ITEMS, e = i - f * Cp::ITEMS;
+            const int g = fq[f];
+            const bool ok = g >= 0 && aok;
+            Cp::run(dst + f * XS, ok ? src + ((size_t)g * d.NA + atom) * nel : src, e, ok);
+        }
+    };
+    auto issue_Y = [&](int tile, int s) {
+        const int b = nbr[(size_t)a * d.NB + s];
+        issue_one(sY, sF + (tile & 1) * 2 * F + F, Y_hat, b, b >= 0 && b < d.NA);
+        tile_cp_commit();
+    };
+
+    if (ODD)  // padding rows and columns stay zero (the copies never write them)
+        for (int i = tid; i < F * XS; i += nt) sX[i] = sY[i] = 0.f;
     if (tid == 0 && t == 0)
         for (int s = 0; s < d.NB; ++s) {
             const int b = nbr[(size_t)a * d.NB + s];
             if (b < 0 || b >= d.NA) atomicOr(status, DEV_BAD_NEIGHBOUR);
         }
+    freq_table(tile0);
+    if (resident)
+        for (int s = 0; s < d.NB; ++s) stage_A(s, s);
+    __syncthreads();
+    if (tile0 < tile1) {
+        issue_one(sX, sF + (tile0 & 1) * 2 * F, X_hat, a, true);
+        issue_Y(tile0, 0);
+    }
 
-    for (size_t i0 = i_begin; i0 < i_end; i0 += c.F) {
-        const bool act = lane && i0 + fl < i_end;
-        const size_t f = act ? freq_of(fm, i0 + fl) : 0;
-        const size_t fneg = act ? freq_neg(fm, f) : 0;
-        __syncthreads();  // the previous batch is done with sX and sSelf
-        if (lane) {
-            float* Xp = sX + (size_t)fl * c.xs;
-#pragma unroll
-            for (int dm = 0; dm < 2; ++dm)
-#pragma unroll
-                for (int dn = 0; dn < 2; ++dn) {
-                    const int m = m0 + dm, n = n0 + dn;
-                    float2 x = make_float2(0.f, 0.f);
-                    if (act && m < Norb && n < Norb) x = X_hat[(f * d.NA + a) * nel + m * Norb + n];
-                    Xp[m * Np + n] = x.x;
-                    Xp[pl + m * Np + n] = x.y;
-                }
-        }
-        for (int g = tid; g < c.F * 9; g += blockDim.x) sSelf[g] = make_float2(0.f, 0.f);
+    for (int tile = tile0; tile < tile1; ++tile) {
         for (int s = 0; s < d.NB; ++s) {
-            const int b = nbr[(size_t)a * d.NB + s];
-            const bool bok = b >= 0 && b < d.NA;
-            if (lane) {
-                float* Yp = sY + (size_t)fl * c.xs;
-#pragma unroll
-                for (int dm = 0; dm < 2; ++dm)
-#pragma unroll
-                    for (int dn = 0; dn < 2; ++dn) {
-                        const int m = m0 + dm, n = n0 + dn;
-                        float2 y = make_float2(0.f, 0.f);
-                        if (act && bok && m < Norb && n < Norb) y = Y_hat[(fneg * d.NA + b) * nel + m * Norb + n];
-                        Yp[m * Np + n] = y.x;
-                        Yp[pl + m * Np + n] = y.y;
-                    }
+            tile_cp_wait();
+            __syncthreads();  // X and Y have landed; the previous bond's sums over sP are done
+            if (s == 0 && tile + 1 < tile1) freq_table(tile + 1);  // read after the next barrier
+            if (!resident) {
+                stage_A(s, 0);
+                __syncthreads();
             }
-            __syncthreads();
-            const float* A = sA + (size_t)s * 12 * pl;
-            // P_i[m][n] = sum_l conj(A_i[l][m]) X[l][n];  R_j[m][n] = sum_l A_j[m][l] Y[l][n] (= AT_j[l][m])
-            float pr[3][4] = {}, pim[3][4] = {};
             if (lane) {
-                const float* Xp = sX + (size_t)fl * c.xs;
-                const float* Yp = sY + (size_t)fl * c.xs;
-                float rr[3][4] = {}, ri[3][4] = {};
-                for (int l = 0; l < Norb; ++l) {
-                    const float2 xr = ld2(Xp + l * Np + n0), xi = ld2(Xp + pl + l * Np + n0);
-                    const float2 yr = ld2(Yp + l * Np + n0), yi = ld2(Yp + pl + l * Np + n0);
+                const float* P = sA + (size_t)(resident ? s : 0) * 2 * S::AB + mp * 4;
+                const float* R = sA + (size_t)(resident ? s : 0) * 2 * S::AB + S::AB + np * 4;
+                const float* X = sX + fs * XS + np * 4;
+                const float* Y = sY + fs * XS + mp * 4;
+                float2 pr[NF][3][2], pi[NF][3][2];  // (P[m0][n], P[m0 + 1][n])
+                float2 rr[NF][3][2], ri[NF][3][2];  // (R[n0][m], R[n0 + 1][m])
 #pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        const float* Ai = A + (size_t)i * 4 * pl;
-                        cmac2x2<true, false>(pr[i], pim[i], ld2(Ai + l * Np + m0), ld2(Ai + pl + l * Np + m0), xr, xi);
-                        cmac2x2<false, false>(rr[i], ri[i], ld2(Ai + 2 * pl + l * Np + m0),
-                                              ld2(Ai + 3 * pl + l * Np + m0), yr, yi);
-                    }
-                }
+                for (int f = 0; f < NF; ++f)
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    float* Rp = sR + (size_t)fl * c.rs + (size_t)j * 2 * pl;
+                    for (int i = 0; i < 3; ++i)
 #pragma unroll
-                    for (int dn = 0; dn < 2; ++dn) {  // transposed: (R[m0][n], R[m0+1][n]) at row n
-                        const int o = (n0 + dn) * Np + m0;
-                        st2(Rp + o, rr[j][dn], rr[j][2 + dn]);
-                        st2(Rp + pl + o, ri[j][dn], ri[j][2 + dn]);
-                    }
-                }
-            }
-            __syncthreads();
-            // this tile's part of C_ij = sum_{m,n} P_i[m][n] R_j[n][m] = sum_{m,n} P_i[m][n] RT_j[m][n]
-            float hp[9][2];
-            if (lane) {
+                        for (int n = 0; n < 2; ++n)
+                            pr[f][i][n] = pi[f][i][n] = rr[f][i][n] = ri[f][i][n] = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int l = 0; l < N; ++l) {
+                    float4 x[NF], y[NF];
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const float* Rp = sR + (size_t)fl * c.rs + (size_t)j * 2 * pl;
-                    float tr[4], ti[4];
-#pragma unroll
-                    for (int dm = 0; dm < 2; ++dm) {
-                        const float2 r2 = ld2(Rp + (m0 + dm) * Np + n0), i2 = ld2(Rp + pl + (m0 + dm) * Np + n0);
-                        tr[dm * 2] = r2.x;
-                        tr[dm * 2 + 1] = r2.y;
-                        ti[dm * 2] = i2.x;
-                        ti[dm * 2 + 1] = i2.y;
+                    for (int f = 0; f < NF; ++f) {
+                        x[f] = lds4(X + f * S::FG * XS + l * NP * 2);
+                        y[f] = lds4(Y + f * S::FG * XS + l * NP * 2);
                     }
 #pragma unroll
                     for (int i = 0; i < 3; ++i) {
-                        float hr = 0.f, hi = 0.f;
+                        const float4 u = lds4(P + (i * NP + l) * S::TN * 4), v = lds4(R + (i * NP + l) * S::TN * 4);
+                        const float2 ar = lo2(u), ai = hi2(u), na = make_float2(-u.z, -u.w);
+                        const float2 br = lo2(v), bi = hi2(v), nb = make_float2(-v.z, -v.w);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            hr = fmaf(pr[i][q], tr[q], hr);
-                            hr = fmaf(-pim[i][q], ti[q], hr);
-                            hi = fmaf(pr[i][q], ti[q], hi);
-                            hi = fmaf(pim[i][q], tr[q], hi);
+                        for (int f = 0; f < NF; ++f)
+#pragma unroll
+                            for (int n = 0; n < 2; ++n) {
+                                const float2 xr = f2dup(n ? x[f].z : x[f].x), xi = f2dup(n ? x[f].w : x[f].y);
+                                const float2 yr = f2dup(n ? y[f].z : y[f].x), yi = f2dup(n ? y[f].w : y[f].y);
+                                pr[f][i][n] = fma2(ar, xr, pr[f][i][n]);  // conj(dH_i[l][m]) X[l][n]
+                                pi[f][i][n] = fma2(ar, xi, pi[f][i][n]);
+                                rr[f][i][n] = fma2(br, yr, rr[f][i][n]);  // dH_j[n][l] Y[l][m]
+                                ri[f][i][n] = fma2(br, yi, ri[f][i][n]);
+                                pr[f][i][n] = fma2(ai, xi, pr[f][i][n]);
+                                pi[f][i][n] = fma2(na, xr, pi[f][i][n]);
+                                rr[f][i][n] = fma2(nb, yi, rr[f][i][n]);
+                                ri[f][i][n] = fma2(bi, yr, ri[f][i][n]);
+                            }
+                    }
+                }
+                // this thread's part of tr(P_i R_j)
+#pragma unroll
+                for (int f = 0; f < NF; ++f) {
+                    float2* o = sP + (size_t)(fs + f * S::FG) * 9 * S::TP + tt;
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) {
+                        float2 qr[2], qi[2];  // (R[n][m0], R[n][m0 + 1])
+                        qr[0] = make_float2(rr[f][j][0].x, rr[f][j][1].x);
+                        qr[1] = make_float2(rr[f][j][0].y, rr[f][j][1].y);
+                        qi[0] = make_float2(ri[f][j][0].x, ri[f][j][1].x);
+                        qi[1] = make_float2(ri[f][j][0].y, ri[f][j][1].y);
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) {
+                            float2 h = make_float2(0.f, 0.f), g = h, k = h;
+#pragma unroll
+                            for (int n = 0; n < 2; ++n) {
+                                h = fma2(pr[f][i][n], qr[n], h);
+                                g = fma2(pi[f][i][n], qi[n], g);
+                                k = fma2(pr[f][i][n], qi[n], k);
+                                k = fma2(pi[f][i][n], qr[n], k);
+                            }
+                            o[(i * 3 + j) * S::TP] = make_float2((h.x + h.y) - (g.x + g.y), k.x + k.y);
                         }
-                        hp[i * 3 + j][0] = hr;
-                        hp[i * 3 + j][1] = hi;
                     }
                 }
             }
-            __syncthreads();  // every read of sR and sY for this bond is done
-            float2* sP = reinterpret_cast<float2*>(sR);  // [F][T][9] trace parts (fit in the R_j planes)
-            if (lane)
-#pragma unroll
-                for (int ij = 0; ij < 9; ++ij) sP[((size_t)fl * T + tt) * 9 + ij] = make_float2(hp[ij][0], hp[ij][1]);
-            __syncthreads();
-            for (int g = tid; g < c.F * 9; g += blockDim.x) {  // fixed-order sums over the tile threads
-                const int rf = g / 9, ij = g - rf * 9;
-                float2 sum = sP[(size_t)rf * T * 9 + ij];
-                for (int u = 1; u < T; ++u) {
-                    const float2 v = sP[((size_t)rf * T + u) * 9 + ij];
-                    sum.x += v.x;
-                    sum.y += v.y;
-                }
-                const float2 self = make_float2(sSelf[g].x + sum.x, sSelf[g].y + sum.y);
-                sSelf[g] = self;
-                if (i0 + rf < i_end) {
-                    const size_t ff = freq_of(fm, i0 + rf);
-                    C_hat[((ff * nA + la) * slots + s) * 9 + ij] = sum;
-                    if (s == d.NB - 1) C_hat[((ff * nA + la) * slots + d.NB) * 9 + ij] = self;
-                }
+            __syncthreads();  // the trace parts are complete; X and Y are free
+            if (s + 1 < d.NB) {
+                issue_Y(tile, s + 1);
+            } else if (tile + 1 < tile1) {
+                issue_one(sX, sF + ((tile + 1) & 1) * 2 * F, X_hat, a, true);
+                issue_Y(tile + 1, 0);
             }
-            // the next bond writes sY before its first barrier and sR (sP) only after it
+            for (int g = tid; g < F * 9; g += nt) {  // fixed-order sums over the tile's threads
+                const int rf = g / 9, ij = g - rf * 9;
+                const int ff = sF[(tile & 1) * 2 * F + rf];
+                if (ff < 0) continue;
+                const float2* v = sP + (size_t)g * S::TP;
+                float2 sum = make_float2(0.f, 0.f), odd = sum;
+#pragma unroll
+                for (int u = 0; u < S::T; u += 2) {
+                    sum = cadd(sum, v[u]);
+                    if (u + 1 < S::T) odd = cadd(odd, v[u + 1]);
+                }
+                sum = cadd(sum, odd);
+                const float2 self = s == 0 ? sum : cadd(sSelf[g], sum);
+                sSelf[g] = self;  // entry g belongs to one thread for the whole tile
+                C_hat[(((size_t)ff * nA + la) * slots + s) * 9 + ij] = sum;
+                if (s == d.NB - 1) C_hat[(((size_t)ff * nA + la) * slots + d.NB) * 9 + ij] = self;
+            }
         }
+    }
+}
+
+template <int NP, int ODD>
+cudaError_t launch_pi32_t(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, const double2* dH,
+                          const float2* const* Gh, float2* const* Ch, unsigned* status, cudaStream_t st) {
+    const PiTileCfg c = make_pi_tile_cfg<NP>(d, fm.count);
+    auto kern = spec_pi32_kernel<NP, ODD>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)(d.a_end - d.a_begin), (unsigned)c.nchunks, 2);
+    SSE_TIMED("spec_pi_kernel", st,
+              kern<<<grid, PiShape<NP>::THREADS, c.smem, st>>>(c, d, fm, nbr, dH, Gh[0], Gh[1], Ch[0], Ch[1], status));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pi32(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, const double2* dH,
+                        const float2* const* Gh, float2* const* Ch, unsigned* status, cudaStream_t st) {
+    switch (d.Norb) {
+#define SSE_PI32(n) \
+    case n: return launch_pi32_t<(n + 1) / 2 * 2, n % 2>(d, fm, nbr, dH, Gh, Ch, status, st);
+        SSE_PI32(1) SSE_PI32(2) SSE_PI32(3) SSE_PI32(4) SSE_PI32(5) SSE_PI32(6) SSE_PI32(7) SSE_PI32(8)
+        SSE_PI32(9) SSE_PI32(10) SSE_PI32(11) SSE_PI32(12) SSE_PI32(13) SSE_PI32(14) SSE_PI32(15) SSE_PI32(16)
+#undef SSE_PI32
+        default: return cudaErrorNotSupported;
     }
 }
 
@@ -446,8 +509,7 @@ size_t spectral_pi32_workspace(const sse_dims& d) { return pi_layout(d, 8).total
 bool spectral_pi_supported(const sse_dims& d) {
     const int L = spectral_length(d);
     return d.Nkz <= kMaxNk && L < kFftMaxLength && make_plan(L).smem <= 227 * 1024 && d.NB <= 16 &&
-           make_pi_cfg(d, (size_t)d.Nkz * L).smem <= 227 * 1024 &&
-           make_pi32_cfg(d, (size_t)d.Nkz * L).smem <= 227 * 1024;
+           make_pi_cfg(d, (size_t)d.Nkz * L).smem <= 227 * 1024;  // the FP32 kernel's limits are wider
 }
 
 namespace {
@@ -490,14 +552,8 @@ cudaError_t spectral_pi_t(const sse_dims& d, const int32_t* nbr, const double2* 
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     if constexpr (fp32) {
-        const Pi32Cfg pc = make_pi32_cfg(d, fm.count);
-        if ((e = cudaFuncSetAttribute(spec_pi32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pc.smem)) !=
-            cudaSuccess)
-            return e;
-        const size_t gy = (fm.count + pc.fchunk - 1) / pc.fchunk;
-        SSE_TIMED("spec_pi_kernel", st,
-                  spec_pi32_kernel<<<dim3((unsigned)nA, (unsigned)gy, 2), pc.threads, pc.smem, st>>>(
-                      pc, d, fm, nbr, dH, Gh[0], Gh[1], Ch[0], Ch[1], status));
+        const float2* Gc[2] = {Gh[0], Gh[1]};
+        if ((e = launch_pi32(d, fm, nbr, dH, Gc, Ch, status, st)) != cudaSuccess) return e;
     } else {
         const PiCfg pc = make_pi_cfg(d, fm.count);
         if ((e = cudaFuncSetAttribute(spec_pi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, pc.smem)) !=
