@@ -120,11 +120,11 @@ size_t fp64_fwd_workspace(const sse_dims&) { return 0; }
 
 cudaError_t fp64_fwd(const Problem& p, double2* S_less, double2* S_greater, unsigned* status, void*, size_t,
                      cudaStream_t st) {
-    const TileCfg c = make_tile_cfg(p.d, kEpiBlocks);
+    const int nA = p.d.a_end - p.d.a_begin;
+    const TileCfg c = make_tile_cfg(p.d, kEpiBlocks, (size_t)p.d.Nkz * 2 * nA);
     if (c.smem > 227 * 1024) return cudaErrorNotSupported;
     cudaError_t e = cudaFuncSetAttribute(sigma_fp64_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, c.smem);
     if (e != cudaSuccess) return e;
-    const int nA = p.d.a_end - p.d.a_begin;
     dim3 grid((p.d.NE + c.TE - 1) / c.TE, p.d.Nkz, 2 * nA);
     SSE_TIMED("sigma_fp64_fwd_kernel", st, sigma_fp64_fwd_kernel<<<grid, c.nthreads, c.smem, st>>>(p, c, S_less, S_greater, status));
     return cudaGetLastError();

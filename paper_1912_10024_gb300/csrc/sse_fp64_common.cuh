@@ -40,7 +40,8 @@ struct TileCfg {
 };
 
 // epi_blocks: complex Norb x Norb blocks per energy that the kernel's epilogue keeps in shared memory.
-inline TileCfg make_tile_cfg(const sse_dims& d, int epi_blocks) {
+// per_tile: CTAs per energy tile where the tiles are a grid dimension, 0 where a CTA walks over all of them.
+inline TileCfg make_tile_cfg(const sse_dims& d, int epi_blocks, size_t per_tile = 0) {
     TileCfg c{};
     c.nel = d.Norb * d.Norb;
     c.P = kMaxThreads / c.nel;
@@ -48,6 +49,11 @@ inline TileCfg make_tile_cfg(const sse_dims& d, int epi_blocks) {
     const int pmax = (kSmemBudget - reserve) / (epi_blocks * kR * c.nel * 16);
     if (c.P > pmax) c.P = pmax;
     if (c.P < 1) c.P = 1;
+    if (per_tile) {
+        // Small problems: see spread_over_fp64. A smaller tile reads more halo rows.
+        c.P = spread_over_fp64(
+            c.P, c.nel, [&](int P) { return per_tile * (size_t)((d.NE + P * kR - 1) / (P * kR)); });
+    }
     c.nthreads = c.P * c.nel;
     c.TE = c.P * kR;
     const int a_bytes = 3 * c.nel * 16;

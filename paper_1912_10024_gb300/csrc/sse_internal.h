@@ -51,6 +51,23 @@ void prof_end(cudaStream_t st);
 int abi_common_checks(const sse_dims* d, const int32_t* nbr, const double* dH, const double* Dl, const double* Dg,
                       const double* Gl, const double* Gg, double scale, int mode, uint32_t flags);
 
+// Work units (frequencies, energy groups) per CTA of the FP64 kernels, `most` at most; nel threads per unit, ctas(u) CTAs
+// at u units. With fewer CTAs than four per SM the fullest SM's FP64 pipe sets the time, so smaller CTAs are taken where
+// they leave that SM at least an eighth fewer warps (whole warps issue); the largest of the sizes that come close stays,
+// since smaller CTAs stage more per unit. Tiny structure, against the largest CTAs: Sigma's direct kernel 680 -> 369 us
+// (24 -> 4 energy pairs; 8 pairs 452 us), Sigma's transform products 76 -> 62 us (32 -> 12 frequencies), the gradient in
+// G likewise 78 -> 63 us; the adjoint, which takes
+// one bond per CTA as well, 232 -> 137 us.
+template <class Ctas>
+int spread_over_fp64(int most, int nel, Ctas ctas) {
+    const auto warps = [&](int u) { return ((ctas(u) + 151) / 152) * (size_t)((u * nel + 31) / 32); };
+    if (ctas(most) >= 4 * 152) return most;
+    int best = most;
+    for (int u = most - 1; u >= 1; --u)
+        if (warps(u) * 8 < warps(best) * 7) best = u;
+    return best;
+}
+
 // Workspace layout: [0, 256) status word + padding; the rest per mode.
 constexpr size_t kStatusBytes = 256;
 

@@ -509,6 +509,11 @@ int pick_frequencies(int nel, SmemOf smem_of, int regs = 64, int max_threads = k
     return best;
 }
 
+// frequencies per CTA of the FP64 product kernels (one batch each in a small problem): see spread_over_fp64
+inline int spread_frequencies(int F, int nel, size_t targets, size_t nfreq) {
+    return spread_over_fp64(F, nel, [&](int f) { return targets * ((nfreq + f - 1) / f); });
+}
+
 struct ProdCfg {
     int nel, F, threads, fchunk;
     int off_A, off_G, off_K, off_W, off_U, smem;
@@ -522,6 +527,7 @@ inline ProdCfg make_prod_cfg(const sse_dims& d, size_t nfreq, int tsz = 8) {
     c.F = pick_frequencies(c.nel, [&](int F) {
         return (long)a16(a16(a16(a16(d.NB * 3 * pl) + F * pl) + F * 9 * 2 * tsz) + F * 3 * pl) + F * 3 * pl;
     });
+    c.F = spread_frequencies(c.F, c.nel, (size_t)(d.a_end - d.a_begin), nfreq);
     c.threads = ((c.F * c.nel + 31) / 32) * 32;
     c.off_A = 0;                                   // [NB][3][planes]
     c.off_G = a16(c.off_A + d.NB * 3 * pl);        // [F][planes]

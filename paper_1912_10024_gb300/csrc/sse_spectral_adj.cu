@@ -16,7 +16,7 @@ namespace {
 // K^ the transformed lag kernel of the forward (c = i*scale).
 // ---------------------------------------------------------------------------
 struct AdjCfg {
-    int nel, F, threads, fchunk, nchunks;
+    int nel, F, threads, fchunk, nchunks, spc;  // spc: bonds per CTA (grid z covers the rest)
     int off_A, off_W, off_G, off_K, off_T, off_V, off_Q, off_D, smem;
 };
 
@@ -43,6 +43,7 @@ AdjCfg make_adj_cfg(const sse_dims& d, size_t nfreq, int tsz = 8) {
         if (useful > best) best = useful, c.F = F;
         (void)threads;
     }
+    c.F = spread_frequencies(c.F, c.nel, (size_t)(d.a_end - d.a_begin) * d.NB, nfreq);
     c.threads = ((c.F * c.nel + 31) / 32) * 32;
     c.off_A = 0;                                   // [3][4 planes: re, im, re+im, re-im] of the current bond
     c.off_W = a16(c.off_A + 3 * 4 * pl);           // [F][4 planes]
@@ -61,6 +62,7 @@ AdjCfg make_adj_cfg(const sse_dims& d, size_t nfreq, int tsz = 8) {
     fc = ((fc + c.F - 1) / c.F) * c.F;
     c.fchunk = (int)(fc < 1 ? 1 : fc);
     c.nchunks = (int)((nfreq + c.fchunk - 1) / c.fchunk);
+    c.spc = nA * c.nchunks < (size_t)152 * 4 ? 1 : d.NB;  // few CTAs: one bond each
     return c;
 }
 
@@ -101,7 +103,7 @@ spec_adj_kernel(AdjCfg c, sse_dims d, const int32_t* __restrict__ nbr, const dou
     const bool lane = fl < c.F;
     const int ndiag = c.F * 9 * Norb;
 
-    for (int s = 0; s < d.NB; ++s) {
+    for (int s = blockIdx.z * c.spc; s < min(d.NB, (int)(blockIdx.z + 1) * c.spc); ++s) {
         const int b = nbr[(size_t)a * d.NB + s];
         const bool bok = b >= 0 && b < d.NA;
         if (!bok && tid == 0) atomicOr(status, DEV_BAD_NEIGHBOUR);
@@ -848,7 +850,8 @@ cudaError_t spectral_bwd_t(const Problem& p, const double2* gS_less, const doubl
                           ac32, d, p.nbr, p.dH, Wh, Gh, Kh, Hh, part + (size_t)t * part_one, L, p.scale, status));
         } else {
             SSE_TIMED("spec_adj_kernel", st,
-                      spec_adj_kernel<T><<<dim3((unsigned)nA, (unsigned)ac.nchunks), ac.threads, ac.smem, st>>>(
+                      spec_adj_kernel<T><<<dim3((unsigned)nA, (unsigned)ac.nchunks, (unsigned)((d.NB + ac.spc - 1) / ac.spc)),
+                                         ac.threads, ac.smem, st>>>(
                           ac, d, p.nbr, p.dH, Wh, Gh, Kh, Hh, part + (size_t)t * part_one, L, p.scale, status));
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -19,6 +19,7 @@ PiCfg make_pi_cfg(const sse_dims& d, size_t nfreq) {
     c.F = pick_frequencies(c.nel, [&](int F) {
         return (long)d.NB * 3 * 4 * pl + F * 3 * pl * 2 + F * 6 * pl * 2 + F * 9 * d.Norb * 16 + F * 9 * 16 + 96;
     });
+    c.F = spread_frequencies(c.F, c.nel, 2 * (size_t)(d.a_end - d.a_begin), nfreq);
     c.threads = ((c.F * c.nel + 31) / 32) * 32;
     c.off_A = 0;                                     // [NB][3][4 planes: re, im, re+im, re-im]
     c.off_X = a16(c.off_A + d.NB * 3 * 4 * pl);      // [F][3 planes]
