@@ -10,7 +10,7 @@
 // (128 bytes per clock and SM, also for a broadcast: a 16-byte load by a warp takes 4 clocks, the issue time of 16
 // warp-wide FMAs). A thread therefore owns half of the rows and two columns of the block, for the three j together and
 // for NF frequencies: at Np = 10 P takes 7.5 FMAs and acc 4.4 per float loaded, against 2 on 2 x 2 tiles for the P_j one
-// frequency at a time. FinFET workload, per step of two types: 52.3 -> 37.2 ms (0.61 of the FP32 pipe; ncu at the
+// frequency at a time. FinFET workload, per step of two types: 52.3 -> 36.6 ms (0.62 of the FP32 pipe; ncu at the
 // adjoint workload: FMA pipe 62% active with the inner loops rolled, shared-memory wavefronts 47%, two warps per
 // scheduler waiting on fixed latencies).
 #pragma once
@@ -32,6 +32,11 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
         : "=f"(d.x), "=f"(d.y)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return d;
+}
+
+// -a on the integer pipe (the FMA pipe is the busy one)
+__device__ __forceinline__ float2 f2neg(float a, float b) {
+    return make_float2(__uint_as_float(__float_as_uint(a) ^ 0x80000000u), __uint_as_float(__float_as_uint(b) ^ 0x80000000u));
 }
 
 __device__ __forceinline__ float4 lds4(const float* p) { return *reinterpret_cast<const float4*>(p); }
@@ -69,11 +74,11 @@ struct TileShape {
     static constexpr int RH = NP / 2;               // rows per thread
     static constexpr int CP = NP / 2;               // column pairs
     static constexpr int TPF = 2 * CP;              // threads per frequency set
-    static constexpr int NF = NP <= 10 ? 2 : 1;     // frequencies per thread: two while their tiles fit in registers
+    static constexpr int NF = NP <= 8 ? 2 : 1;      // frequencies per thread: two while their tiles fit in registers
     // CTAs per SM that the registers (P 12 Np NF / 2, acc 2 Np NF, operands) leave room for without spills. Measured at
-    // Norb = 10: NF = 2 with two CTAs 37.2 ms per FinFET step, NF = 1 with three 37.7, with four (spills) 45.8; at
-    // Norb = 12 (gradient in G, NA = 200): NF = 1 with three CTAs 3.9 ms, with two 4.2.
-    static constexpr int CTAS = NP <= 4 ? 4 : NP == 6 || NP == 12 ? 3 : 2;
+    // Norb = 10: NF = 1 with three CTAs 36.6 ms per FinFET step, NF = 2 with two 37.1, NF = 1 with four (spills) 45.8; at
+    // Norb = 12 (gradient in G, NA = 200): NF = 1 with three CTAs 3.8 ms, with two 4.2.
+    static constexpr int CTAS = NP <= 4 ? 4 : NP == 6 || NP == 10 || NP == 12 ? 3 : 2;
     static constexpr int XS = NP * NP * 2;          // floats of X per frequency
     static constexpr int US = 3 * NP * NP * 2;      // floats of U per frequency
     static constexpr int RSTR = (NP + 1) * 4;       // floats per column pair of the right operand (odd: bank spread)
@@ -265,7 +270,7 @@ __global__ void __launch_bounds__(128, TileShape<NP>::CTAS) spec_prod32_kernel(T
 #pragma unroll
                         for (int j = 0; j < 3; ++j) {
                             const float4 b = lds4(R + j * CP * S::RSTR + (l + dl) * 4);
-                            const float2 br = lo2(b), bi = hi2(b);
+                            const float2 br = lo2(b), bi = hi2(b), nbi = f2neg(b.z, b.w);
 #pragma unroll
                             for (int f = 0; f < NF; ++f)
 #pragma unroll
@@ -273,7 +278,7 @@ __global__ void __launch_bounds__(128, TileShape<NP>::CTAS) spec_prod32_kernel(T
                                     const float x = dl ? g[f][r].z : g[f][r].x, y = dl ? g[f][r].w : g[f][r].y;
                                     pr[f][j][r] = fma2(f2dup(x), br, pr[f][j][r]);
                                     pi[f][j][r] = fma2(f2dup(x), bi, pi[f][j][r]);
-                                    pr[f][j][r] = fma2(f2dup(-y), bi, pr[f][j][r]);
+                                    pr[f][j][r] = fma2(f2dup(y), nbi, pr[f][j][r]);
                                     pi[f][j][r] = fma2(f2dup(y), br, pi[f][j][r]);
                                 }
                         }
@@ -327,13 +332,13 @@ __global__ void __launch_bounds__(128, TileShape<NP>::CTAS) spec_prod32_kernel(T
 #pragma unroll
                             for (int f = 0; f < NF; ++f) {
                                 const float4 u = lds4(U + (size_t)f * c.fg * S::US + (i * NP + m + dm) * CP * 4);
-                                const float2 ur = lo2(u), ui = hi2(u);
+                                const float2 ur = lo2(u), ui = hi2(u), nui = f2neg(u.z, u.w);
 #pragma unroll
                                 for (int r = 0; r < RH; ++r) {
                                     const float x = dm ? t[r].z : t[r].x, y = dm ? t[r].w : t[r].y;
                                     ar[f][r] = fma2(f2dup(x), ur, ar[f][r]);
                                     ai[f][r] = fma2(f2dup(x), ui, ai[f][r]);
-                                    ar[f][r] = fma2(f2dup(-y), ui, ar[f][r]);
+                                    ar[f][r] = fma2(f2dup(y), nui, ar[f][r]);
                                     ai[f][r] = fma2(f2dup(y), ur, ai[f][r]);
                                 }
                             }

@@ -350,8 +350,8 @@ spec_pi32_kernel(PiTileCfg c, sse_dims d, FreqMap fm, const int32_t* __restrict_
 #pragma unroll
                     for (int i = 0; i < 3; ++i) {
                         const float4 u = lds4(P + (i * NP + l) * S::TN * 4), v = lds4(R + (i * NP + l) * S::TN * 4);
-                        const float2 ar = lo2(u), ai = hi2(u), na = make_float2(-u.z, -u.w);
-                        const float2 br = lo2(v), bi = hi2(v), nb = make_float2(-v.z, -v.w);
+                        const float2 ar = lo2(u), ai = hi2(u), na = f2neg(u.z, u.w);
+                        const float2 br = lo2(v), bi = hi2(v), nb = f2neg(v.z, v.w);
 #pragma unroll
                         for (int f = 0; f < NF; ++f)
 #pragma unroll
