@@ -1,12 +1,9 @@
-// Transform kernels with compile-time sizes. (1) FP32 E-direction transforms with the DFT codelets in registers,
-// for the transform lengths of the stated workloads and of the small test shapes: each CTA transforms 8 adjacent
-// columns of one batch, of length L = L1 * L2, as two passes over a tile in shared memory (the four-step
-// factorisation of the DFT: L2 DFTs of length L1 down the stride-L2 rows, the twiddles exp(-2 pi i n2 k1 / L), then
-// L1 DFTs of length L2 along contiguous rows, both in place), and stores the frequencies in natural order. Every index
-// inside a codelet is a constant; the radix-4/2/3 Stockham kernel fft_e_kernel keeps every other length and the FP64
-// transforms. Same loader and store interface. At the FinFET workload (L = 576) the transform of G takes 2.9 ms per
-// type against 3.8 ms for fft_e_kernel (2.6 ms with the prefetching variant below), the inverse transform into
-// Sigma 2.3 ms against 3.2. (2) The kz DFT of FP32 and FP64 spectra with the grid size as a template parameter.
+// Transform kernels with compile-time sizes. (1) FP32 E-direction transforms with the DFT codelets in registers: each CTA
+// transforms 8 adjacent columns of one batch, of length L = L1 * L2, in two passes (the four-step factorisation of the
+// DFT: L2 DFTs of length L1 down the stride-L2 rows, the twiddles exp(-2 pi i n2 k1 / L), then L1 DFTs of length L2 along
+// contiguous rows) with one exchange through shared memory. Every index inside a codelet is a constant; the radix-4/2/3
+// Stockham kernel fft_e_kernel keeps the lengths without two codelet factors and the FP64 transforms. Same loader and
+// store interface. (2) The kz DFT of FP32 and FP64 spectra with the grid size as a template parameter.
 //
 // Included at the end of sse_spectral.cuh (it uses that file's loaders, stores, CT, launch_fft and SSE_TIMED).
 #pragma once
@@ -138,101 +135,122 @@ struct RegDft {
     }
 };
 
-constexpr int kE4Cols = 8;        // columns per CTA: 128-byte rows of FP64 input, 64-byte rows of FP32
-constexpr int kE4Threads = 256;
-constexpr int kE4LoadBatch = 8;   // global loads in flight per thread while the tile is read
+constexpr int kE4Cols = 8;  // columns per CTA: 128-byte rows of FP64 input, 64-byte rows of FP32
 
-template <int L1, int L2>
-struct E4Shape {
-    static constexpr int L = L1 * L2;
-    static constexpr int P = (L2 % 2 == 0) ? 1 : 0;  // a block of L2 rows padded to an odd count (banks)
-    static constexpr int LP = L2 + P;
-    static constexpr int SL = L1 * LP * kE4Cols;     // float2 of the tile
-    static constexpr int SMEM = SL * 8 + L * 8;      // tile + twiddle table
-    // CTAs per SM the register budget is sized for (occupancy, not loads per thread, sets the load throughput):
-    // four (64 registers) up to L = 576, two for the 32 x 36 codelets
-    static constexpr int MIN_CTAS = L <= 576 ? 4 : 2;
-    // position of input row r = L2 n1 + n2, and of output frequency e = k1 + L1 k2 after the two passes
-    __device__ __forceinline__ static int pos_in(int r) { return (r / L2) * LP + r % L2; }
-    __device__ __forceinline__ static int pos_out(int e) { return (e % L1) * LP + e / L1; }
-};
+// codelet lengths: the small set keeps two 24-point columns' worth of registers free for occupancy, the large one reaches
+// L = 36^2
+constexpr int kE4Small = 24, kE4Large = 36;
+inline bool e4_codelet(int n, int most) {
+    for (int c : {4, 6, 8, 9, 12, 16, 18, 24, 27, 32, 36})
+        if (n == c) return n <= most;
+    return false;
+}
 
-// CTA: kE4Cols adjacent columns of one batch (blockIdx.y). ld(batch, r, col) gives row r < L (zero where the loader
-// pads), sv(batch, e, col, v) takes frequency rows e < sv.rows, as for fft_e_kernel.
-template <int L1, int L2, class Load, class Store>
-__global__ void __launch_bounds__(kE4Threads, E4Shape<L1, L2>::MIN_CTAS)
-    fft_e4_kernel(const double2* __restrict__ tw_g, Load ld, Store sv, size_t ncols) {
-    using S = E4Shape<L1, L2>;
-    constexpr int CC = kE4Cols, L = S::L;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* X = reinterpret_cast<float2*>(smem_raw);  // [L1][LP][CC]
-    float2* tw = X + S::SL;                          // [L] exp(-2 pi i m / L)
-    const int tid = threadIdx.x, nt = blockDim.x, batch = blockIdx.y;
-    const size_t col0 = (size_t)blockIdx.x * CC;
-    for (int m = tid; m < L; m += nt) tw[m] = make_float2((float)tw_g[m].x, (float)tw_g[m].y);
-    // 1. the tile, kE4LoadBatch loads in flight per thread
-    constexpr int total = L * CC;
-    for (int b0 = tid; b0 < total; b0 += kE4LoadBatch * nt) {
-        float2 v[kE4LoadBatch];
-#pragma unroll
-        for (int u = 0; u < kE4LoadBatch; ++u) {
-            const int i = b0 + u * nt, c = i % CC, r = i / CC;
-            v[u] = (i < total && col0 + c < ncols) ? ld(batch, r, col0 + c) : make_float2(0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < kE4LoadBatch; ++u) {
-            const int i = b0 + u * nt;
-            if (i < total) X[S::pos_in(i / CC) * CC + i % CC] = v[u];
-        }
-    }
-    __syncthreads();
-    // 2. L2 DFTs of length L1 per column (rows L2 n1 + n2, n1 = 0 .. L1-1), twiddled by w_L^(n2 k1), in place
-    for (int t = tid; t < CC * L2; t += nt) {
-        const int c = t % CC, n2 = t / CC;
-        float2* p = X + n2 * CC + c;
-        float2 x[L1];
-#pragma unroll
-        for (int n1 = 0; n1 < L1; ++n1) x[n1] = p[n1 * S::LP * CC];
-        RegDft<L1>::run(x);
-#pragma unroll
-        for (int k1 = 1; k1 < L1; ++k1) x[k1] = cmul(x[k1], tw[n2 * k1]);
-#pragma unroll
-        for (int k1 = 0; k1 < L1; ++k1) p[k1 * S::LP * CC] = x[k1];
-    }
-    __syncthreads();
-    // 3. L1 DFTs of length L2 along each block of contiguous rows, in place: position L2 k1 + k2 then holds the
-    //    frequency k1 + L1 k2
-    for (int t = tid; t < CC * L1; t += nt) {
-        const int c = t % CC, k1 = t / CC;
-        float2* p = X + k1 * S::LP * CC + c;
-        float2 x[L2];
-#pragma unroll
-        for (int n2 = 0; n2 < L2; ++n2) x[n2] = p[n2 * CC];
-        RegDft<L2>::run(x);
-#pragma unroll
-        for (int k2 = 0; k2 < L2; ++k2) p[k2 * CC] = x[k2];
-    }
-    __syncthreads();
-    // 4. frequencies in natural order
-    for (int t = tid; t < sv.rows * CC; t += nt) {
-        const int c = t % CC, e = t / CC;
-        if (col0 + c < ncols) sv(batch, e, col0 + c, X[S::pos_out(e) * CC + c]);
+// f(std::integral_constant<int, n>) for a codelet length n known at run time
+template <int MOST, class F>
+__device__ __forceinline__ void e4_with(int n, F&& f) {
+    switch (n) {
+        case 4: f(std::integral_constant<int, 4>{}); break;
+        case 6: f(std::integral_constant<int, 6>{}); break;
+        case 8: f(std::integral_constant<int, 8>{}); break;
+        case 9: f(std::integral_constant<int, 9>{}); break;
+        case 12: f(std::integral_constant<int, 12>{}); break;
+        case 16: f(std::integral_constant<int, 16>{}); break;
+        case 18: f(std::integral_constant<int, 18>{}); break;
+        case 24: f(std::integral_constant<int, 24>{}); break;
+        default:
+            if constexpr (MOST > kE4Small) {
+                if (n == 27) f(std::integral_constant<int, 27>{});
+                else if (n == 32) f(std::integral_constant<int, 32>{});
+                else f(std::integral_constant<int, 36>{});
+            }
     }
 }
 
-template <int L1, int L2, class Load, class Store>
-cudaError_t launch_e4_t(const char* name, const double2* tw, Load ld, Store sv, size_t ncols, int batches,
+struct E4Plan {
+    int L, L1, L2, LP;  // L = L1 * L2; blocks of L2 rows padded to LP, an odd count (banks)
+    int threads, smem;  // one thread per column and codelet; tile + twiddle table
+    bool ok, large;
+};
+
+// the most balanced factorisation into two codelet lengths
+inline E4Plan make_e4_plan(int L) {
+    E4Plan p{};
+    p.L = L;
+    for (int a = 4; a * a <= L; ++a)
+        if (L % a == 0 && e4_codelet(a, kE4Large) && e4_codelet(L / a, kE4Large)) p.L1 = a, p.L2 = L / a, p.ok = true;
+    if (!p.ok) return p;
+    p.LP = p.L2 | 1;
+    p.large = p.L2 > kE4Small;
+    p.threads = (kE4Cols * p.L2 + 31) / 32 * 32;
+    p.smem = p.L1 * p.LP * kE4Cols * 8 + L * 8;
+    return p;
+}
+
+// CTA: kE4Cols adjacent columns of one batch (blockIdx.y). ld(batch, r, col) gives row r < L (zero where the loader
+// pads), sv(batch, e, col, v) takes frequency rows e < sv.rows, as for fft_e_kernel. Pass 1 reads its rows from global
+// memory (all rows of a codelet in flight) and pass 2 writes its frequencies there: the tile crosses shared memory once,
+// with one barrier. The codelet lengths are run-time
+// choices inside one kernel, so every L = 2^a 3^b with two factors among them (all from 36 to 576 but a few) is served.
+// FinFET, two types: inverse transform of S^ 4.64 -> 3.84 ms (four barriers and the tile crossing shared memory four times
+// before); L = 324 (NA = 90, Norb = 7): 97 -> 74 us against the Stockham kernel.
+template <int MOST>
+struct E4Bounds {  // at most 192 threads with four CTAs per SM (85 registers), or 288 with two (112)
+    static constexpr int THREADS = (kE4Cols * MOST + 31) / 32 * 32, CTAS = MOST <= kE4Small ? 4 : 2;
+};
+
+template <int MOST, class Load, class Store>
+__global__ void __launch_bounds__(E4Bounds<MOST>::THREADS, E4Bounds<MOST>::CTAS)
+    fft_e4_kernel(E4Plan p, const float2* __restrict__ tw_g, Load ld, Store sv, size_t ncols) {
+    constexpr int CC = kE4Cols;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2* X = reinterpret_cast<float2*>(smem_raw);  // [L1][LP][CC]
+    float2* tw = X + p.L1 * p.LP * CC;               // [L] exp(-2 pi i m / L)
+    const int tid = threadIdx.x, batch = blockIdx.y, c = tid % CC, q = tid / CC;
+    const size_t col = (size_t)blockIdx.x * CC + c;
+    const bool in = col < ncols;
+    for (int m = tid; m < p.L; m += blockDim.x) tw[m] = tw_g[m];
+    // 1. DFTs of length L1 (rows L2 n1 + n2, n2 = q), twiddled by w_L^(n2 k1)
+    e4_with<MOST>(p.L1, [&](auto nc) {
+        constexpr int N = decltype(nc)::value;
+        float2 x[N];
+#pragma unroll
+        for (int n1 = 0; n1 < N; ++n1)
+            x[n1] = in && q < p.L2 ? ld(batch, p.L2 * n1 + q, col) : make_float2(0.f, 0.f);
+        RegDft<N>::run(x);
+        __syncthreads();  // the twiddle table
+        if (q < p.L2) {
+#pragma unroll
+            for (int k1 = 0; k1 < N; ++k1) X[(k1 * p.LP + q) * CC + c] = k1 ? cmul(x[k1], tw[q * k1]) : x[k1];
+        }
+    });
+    __syncthreads();
+    // 2. DFTs of length L2 along each block of contiguous rows (k1 = q): frequency k1 + L1 k2
+    if (q >= p.L1) return;
+    e4_with<MOST>(p.L2, [&](auto nc) {
+        constexpr int N = decltype(nc)::value;
+        float2 x[N];
+#pragma unroll
+        for (int n2 = 0; n2 < N; ++n2) x[n2] = X[(q * p.LP + n2) * CC + c];
+        RegDft<N>::run(x);
+#pragma unroll
+        for (int k2 = 0; k2 < N; ++k2) {
+            const int e = q + p.L1 * k2;
+            if (in && e < sv.rows) sv(batch, e, col, x[k2]);
+        }
+    });
+}
+
+template <int MOST, class Load, class Store>
+cudaError_t launch_e4_t(const char* name, const E4Plan& p, const float2* tw, Load ld, Store sv, size_t ncols, int batches,
                         cudaStream_t st) {
-    using S = E4Shape<L1, L2>;
-    cudaError_t e =
-        cudaFuncSetAttribute(fft_e4_kernel<L1, L2, Load, Store>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
+    auto kern = fft_e4_kernel<MOST, Load, Store>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
     if (e != cudaSuccess) return e;
     const size_t gx = (ncols + kE4Cols - 1) / kE4Cols;
     if (gx == 0 || batches == 0) return cudaSuccess;
     if (gx > 0x7fffffffu || batches > 65535) return cudaErrorInvalidValue;
-    SSE_TIMED(name, st,
-              fft_e4_kernel<L1, L2, Load, Store><<<dim3((unsigned)gx, (unsigned)batches), kE4Threads, S::SMEM, st>>>(
-                  tw, ld, sv, ncols));
+    SSE_TIMED(name, st, kern<<<dim3((unsigned)gx, (unsigned)batches), p.threads, p.smem, st>>>(p, tw, ld, sv, ncols));
     return cudaGetLastError();
 }
 
@@ -281,85 +299,78 @@ __device__ __forceinline__ void cp_async_elem(uint32_t dst, const void* src, boo
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(ok ? 8 : 0) : "memory");
 }
 
-template <int L1, int L2, class Load>
-size_t e4p_smem(const Load& ld) {
-    return (size_t)E4Shape<L1, L2>::SMEM + (size_t)ld.src_rows() * kE4Cols * sizeof(typename Load::Raw);
+template <class Load>
+size_t e4p_smem(const E4Plan& p, const Load& ld) {
+    return (size_t)p.smem + (size_t)ld.src_rows() * kE4Cols * sizeof(typename Load::Raw);
 }
 
-template <int L1, int L2, class Load, class Store>
-__global__ void __launch_bounds__(kE4Threads, 2)
-    fft_e4p_kernel(const double2* __restrict__ tw_g, Load ld, Store sv, size_t ncols, int gx, int ntiles) {
-    using S = E4Shape<L1, L2>;
+template <int MOST, class Load, class Store>
+__global__ void __launch_bounds__(E4Bounds<MOST>::THREADS, MOST <= kE4Small ? 3 : 2)
+    fft_e4p_kernel(E4Plan p, const float2* __restrict__ tw_g, Load ld, Store sv, size_t ncols, int gx, int ntiles) {
     using Raw = typename Load::Raw;
-    constexpr int CC = kE4Cols, L = S::L;
+    constexpr int CC = kE4Cols;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* X = reinterpret_cast<float2*>(smem_raw);  // [L1][LP][CC]
-    float2* tw = X + S::SL;                          // [L]
-    Raw* raw = reinterpret_cast<Raw*>(tw + L);       // [rows][CC]: the next tile as stored (16-byte aligned: L even)
-    const int tid = threadIdx.x, nt = blockDim.x;
     const int rows = ld.src_rows();
+    Raw* raw = reinterpret_cast<Raw*>(smem_raw);                       // [rows][CC]: the next tile as stored
+    float2* X = reinterpret_cast<float2*>(raw + (size_t)rows * CC);  // [L1][LP][CC]
+    float2* tw = X + p.L1 * p.LP * CC;                               // [L]
+    const int tid = threadIdx.x, nt = blockDim.x, c = tid % CC;
+    int q = tid / CC;
     const uint32_t raw_s = (uint32_t)__cvta_generic_to_shared(raw);
     auto issue = [&](int tile) {
         const int batch = tile / gx;
-        const size_t col0 = (size_t)(tile % gx) * CC;
-        for (int i = tid; i < rows * CC; i += nt) {
-            const int c = i % CC, r = i / CC;
-            const bool ok = col0 + c < ncols;
-            cp_async_elem<(int)sizeof(Raw)>(raw_s + (uint32_t)(i * (int)sizeof(Raw)),
-                                           ld.src(ok ? batch : 0, ok ? r : 0, ok ? col0 + c : 0), ok);
-        }
+        const size_t col = (size_t)(tile % gx) * CC + c;
+        const bool ok = col < ncols;
+        for (int r = q; r < rows; r += nt / CC)
+            cp_async_elem<(int)sizeof(Raw)>(raw_s + (uint32_t)((r * CC + c) * (int)sizeof(Raw)),
+                                           ld.src(ok ? batch : 0, ok ? r : 0, ok ? col : 0), ok);
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    for (int m = tid; m < L; m += nt) tw[m] = make_float2((float)tw_g[m].x, (float)tw_g[m].y);
+    for (int m = tid; m < p.L; m += nt) tw[m] = tw_g[m];
     if ((int)blockIdx.x < ntiles) issue(blockIdx.x);
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int batch = tile / gx;
-        const size_t col0 = (size_t)(tile % gx) * CC;
+        const size_t col = (size_t)(tile % gx) * CC + c;
+        asm volatile("" : "+r"(q));  // or the addresses of every codelet length are kept across tiles (and spilled)
         asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();  // the raw tile has landed for every thread; the previous tile's store has read X
-        for (int i = tid; i < L * CC; i += nt) {
-            const int r = i / CC;
-            X[S::pos_in(r) * CC + i % CC] = r < rows ? Load::cvt(raw[i]) : make_float2(0.f, 0.f);
-        }
-        __syncthreads();  // the raw buffer is free
+        __syncthreads();  // the raw tile has landed for every thread; the previous tile's second pass has read X
+        e4_with<MOST>(p.L1, [&](auto nc) {
+            constexpr int N = decltype(nc)::value;
+            if (q >= p.L2) return;
+            float2 x[N];
+#pragma unroll
+            for (int n1 = 0; n1 < N; ++n1) {
+                const int r = p.L2 * n1 + q;
+                x[n1] = r < rows ? Load::cvt(raw[r * CC + c]) : make_float2(0.f, 0.f);
+            }
+            RegDft<N>::run(x);
+#pragma unroll
+            for (int k1 = 0; k1 < N; ++k1) X[(k1 * p.LP + q) * CC + c] = k1 ? cmul(x[k1], tw[q * k1]) : x[k1];
+        });
+        __syncthreads();  // X is complete, the raw buffer is free
         if (tile + (int)gridDim.x < ntiles) issue(tile + gridDim.x);
-        for (int t = tid; t < CC * L2; t += nt) {
-            const int c = t % CC, n2 = t / CC;
-            float2* p = X + n2 * CC + c;
-            float2 x[L1];
+        if (q >= p.L1) continue;
+        e4_with<MOST>(p.L2, [&](auto nc) {
+            constexpr int N = decltype(nc)::value;
+            float2 x[N];
 #pragma unroll
-            for (int n1 = 0; n1 < L1; ++n1) x[n1] = p[n1 * S::LP * CC];
-            RegDft<L1>::run(x);
+            for (int n2 = 0; n2 < N; ++n2) x[n2] = X[(q * p.LP + n2) * CC + c];
+            RegDft<N>::run(x);
 #pragma unroll
-            for (int k1 = 1; k1 < L1; ++k1) x[k1] = cmul(x[k1], tw[n2 * k1]);
-#pragma unroll
-            for (int k1 = 0; k1 < L1; ++k1) p[k1 * S::LP * CC] = x[k1];
-        }
-        __syncthreads();
-        for (int t = tid; t < CC * L1; t += nt) {
-            const int c = t % CC, k1 = t / CC;
-            float2* p = X + k1 * S::LP * CC + c;
-            float2 x[L2];
-#pragma unroll
-            for (int n2 = 0; n2 < L2; ++n2) x[n2] = p[n2 * CC];
-            RegDft<L2>::run(x);
-#pragma unroll
-            for (int k2 = 0; k2 < L2; ++k2) p[k2 * CC] = x[k2];
-        }
-        __syncthreads();
-        for (int t = tid; t < sv.rows * CC; t += nt) {
-            const int c = t % CC, e = t / CC;
-            if (col0 + c < ncols) sv(batch, e, col0 + c, X[S::pos_out(e) * CC + c]);
-        }
+            for (int k2 = 0; k2 < N; ++k2) {
+                const int e = q + p.L1 * k2;
+                if (col < ncols && e < sv.rows) sv(batch, e, col, x[k2]);
+            }
+        });
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-template <int L1, int L2, class Load, class Store>
-cudaError_t launch_e4p_t(const char* name, const double2* tw, Load ld, Store sv, size_t ncols, int batches,
-                         cudaStream_t st) {
-    const size_t smem = e4p_smem<L1, L2>(ld);
-    auto kern = fft_e4p_kernel<L1, L2, Load, Store>;
+template <int MOST, class Load, class Store>
+cudaError_t launch_e4p_t(const char* name, const E4Plan& p, const float2* tw, Load ld, Store sv, size_t ncols,
+                         int batches, cudaStream_t st) {
+    const size_t smem = e4p_smem(p, ld);
+    auto kern = fft_e4p_kernel<MOST, Load, Store>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const size_t gx = (ncols + kE4Cols - 1) / kE4Cols;
@@ -369,41 +380,34 @@ cudaError_t launch_e4p_t(const char* name, const double2* tw, Load ld, Store sv,
     int dev = 0, nsm = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kE4Threads, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, p.threads, smem)) != cudaSuccess) return e;
     const int grid = std::min(ntiles, std::max(1, per_sm) * nsm);
-    SSE_TIMED(name, st, kern<<<grid, kE4Threads, smem, st>>>(tw, ld, sv, ncols, (int)gx, ntiles));
+    SSE_TIMED(name, st, kern<<<grid, p.threads, smem, st>>>(p, tw, ld, sv, ncols, (int)gx, ntiles));
     return cudaGetLastError();
 }
 
-// The prefetching kernel for FP64 input tiles (G: 16-byte elements, the larger share of the transform's traffic)
-// where the staging buffer fits; fft_e4_kernel otherwise. Measured at FinFET (L = 576), per step of two types: the
-// transform of G 5.81 -> 5.27 ms with the prefetch; the inverse transform into Sigma (FP32 spectrum in, 8-byte
-// elements) 4.62 -> 5.05 ms with it (two CTAs per SM instead of four), so it keeps fft_e4_kernel.
-template <int L1, int L2, class Load, class Store>
-cudaError_t launch_e4_any(const char* name, const double2* tw, Load ld, Store sv, size_t ncols, int batches,
-                          cudaStream_t st) {
+// The prefetching kernel for FP64 input tiles where the staging buffer fits: FinFET, transform of G, both types 4.70 ms
+// against 6.22 with fft_e4_kernel (the conversions hold up its loads); fft_e4_kernel for FP32 input, which needs none.
+template <int MOST, class Load, class Store>
+cudaError_t launch_e4_any(const char* name, const E4Plan& p, const float2* tw, Load ld, Store sv, size_t ncols,
+                          int batches, cudaStream_t st) {
     if constexpr (HasRawSrc<Load>::value && sizeof(typename HasRawSrcType<Load>::type) == 16) {
-        if (e4p_smem<L1, L2>(ld) <= (size_t)kE4pSmemMax)
-            return launch_e4p_t<L1, L2>(e4_label(name, true), tw, ld, sv, ncols, batches, st);
+        if (e4p_smem(p, ld) <= (size_t)kE4pSmemMax)
+            return launch_e4p_t<MOST>(e4_label(name, true), p, tw, ld, sv, ncols, batches, st);
     }
-    return launch_e4_t<L1, L2>(e4_label(name, false), tw, ld, sv, ncols, batches, st);
+    return launch_e4_t<MOST>(e4_label(name, false), p, tw, ld, sv, ncols, batches, st);
 }
 
-
-// FP32 E-transforms at the lengths with an instantiation (those of the stated workloads and of the small test
-// shapes); every other length, and the FP64 transforms, take fft_e_kernel.
+// FP32 E-transforms of the lengths with two codelet factors; every other length, and the FP64 transforms, take
+// fft_e_kernel.
 template <class Load, class Store>
-cudaError_t launch_fft32(const char* name, const FftPlan& p, const double2* tw, Load ld, Store sv, size_t ncols,
+cudaError_t launch_fft32(const char* name, const FftPlan& p, const typename Load::C* tw, Load ld, Store sv, size_t ncols,
                          int batches, cudaStream_t st) {
     if constexpr (std::is_same<typename Load::C, float2>::value) {
-        switch (p.L) {
-            case 36: return launch_e4_any<6, 6>(name, tw, ld, sv, ncols, batches, st);
-            case 54: return launch_e4_any<6, 9>(name, tw, ld, sv, ncols, batches, st);
-            case 288: return launch_e4_any<16, 18>(name, tw, ld, sv, ncols, batches, st);
-            case 576: return launch_e4_any<24, 24>(name, tw, ld, sv, ncols, batches, st);
-            case 1152: return launch_e4_any<32, 36>(name, tw, ld, sv, ncols, batches, st);
-            default: break;
-        }
+        const E4Plan e4 = make_e4_plan(p.L);
+        if (e4.ok)
+            return e4.large ? launch_e4_any<kE4Large>(name, e4, tw, ld, sv, ncols, batches, st)
+                            : launch_e4_any<kE4Small>(name, e4, tw, ld, sv, ncols, batches, st);
     }
     return launch_fft(name, p, tw, ld, sv, ncols, batches, st);
 }
@@ -413,56 +417,62 @@ cudaError_t launch_fft32(const char* name, const FftPlan& p, const double2* tw, 
 // the cosines and sines compile-time constants. Inputs k and Nk - k are paired (p = x_k + x_{Nk-k},
 // q = x_k - x_{Nk-k}) and so are outputs kappa and Nk - kappa: out[kappa] = C -+ i S, out[Nk - kappa] = C +- i S
 // with C = x_0 (+ (-1)^kappa x_{Nk/2}) + sum_k p_k cos(2 pi k kappa / Nk), S = sum_k q_k sin(2 pi k kappa / Nk).
-template <class C, int NK>
-__global__ void __launch_bounds__(256) dft_kz_kernel(C* __restrict__ X, int n_in, size_t M, int inverse) {
+// out(kappa, value) takes each result once.
+template <class C, int NK, class Out>
+__device__ __forceinline__ void kz_dft(const C (&x)[NK], int inverse, Out&& out) {
     using R = typename CT<C>::R;
     constexpr int H = (NK - 1) / 2;  // (k, NK - k) pairs
     constexpr bool EVEN = NK % 2 == 0;
     const R sgn = inverse ? (R)1 : (R)-1;
+    C p[H + 1], q[H + 1];
+    C c0 = x[0];
+#pragma unroll
+    for (int k = 1; k <= H; ++k) {
+        p[k] = cadd(x[k], x[NK - k]);
+        q[k] = csub(x[k], x[NK - k]);
+        c0 = cadd(c0, p[k]);
+    }
+    const C xh = EVEN ? x[NK / 2] : CT<C>::mk(0, 0);
+    out(0, cadd(c0, xh));
+    static_for<1, H + 1>([&](auto kc) {
+        constexpr int kap = decltype(kc)::value;
+        C Cs = x[0], Sn = CT<C>::mk(0, 0);
+        static_for<1, H + 1>([&](auto jc) {
+            constexpr int k = decltype(jc)::value;
+            constexpr CxCis w = cx_cis((long)k * kap, NK);
+            Cs.x = fma(p[k].x, (R)w.c, Cs.x);
+            Cs.y = fma(p[k].y, (R)w.c, Cs.y);
+            Sn.x = fma(q[k].x, (R)w.s, Sn.x);
+            Sn.y = fma(q[k].y, (R)w.s, Sn.y);
+        });
+        if constexpr (EVEN) {
+            constexpr R e = (kap & 1) ? (R)-1 : (R)1;
+            Cs.x = fma(e, xh.x, Cs.x);
+            Cs.y = fma(e, xh.y, Cs.y);
+        }
+        out(kap, CT<C>::mk(Cs.x - sgn * Sn.y, Cs.y + sgn * Sn.x));
+        out(NK - kap, CT<C>::mk(Cs.x + sgn * Sn.y, Cs.y - sgn * Sn.x));
+    });
+    if constexpr (EVEN && NK > 1) {  // kappa = NK/2: cos(pi k) = (-1)^k, sin = 0
+        C Cs = x[0];
+#pragma unroll
+        for (int k = 1; k <= H; ++k) {
+            const R e = (k & 1) ? (R)-1 : (R)1;
+            Cs.x = fma(e, p[k].x, Cs.x);
+            Cs.y = fma(e, p[k].y, Cs.y);
+        }
+        constexpr R e = ((NK / 2) & 1) ? (R)-1 : (R)1;
+        out(NK / 2, CT<C>::mk(fma(e, xh.x, Cs.x), fma(e, xh.y, Cs.y)));
+    }
+}
+
+template <class C, int NK>
+__global__ void __launch_bounds__(256) dft_kz_kernel(C* __restrict__ X, int n_in, size_t M, int inverse) {
     for (size_t m = blockIdx.x * (size_t)blockDim.x + threadIdx.x; m < M; m += (size_t)gridDim.x * blockDim.x) {
         C x[NK];
 #pragma unroll
         for (int k = 0; k < NK; ++k) x[k] = k < n_in ? X[(size_t)k * M + m] : CT<C>::mk(0, 0);
-        C p[H + 1], q[H + 1];
-        C c0 = x[0];
-#pragma unroll
-        for (int k = 1; k <= H; ++k) {
-            p[k] = cadd(x[k], x[NK - k]);
-            q[k] = csub(x[k], x[NK - k]);
-            c0 = cadd(c0, p[k]);
-        }
-        const C xh = EVEN ? x[NK / 2] : CT<C>::mk(0, 0);
-        X[m] = cadd(c0, xh);
-        static_for<1, H + 1>([&](auto kc) {
-            constexpr int kap = decltype(kc)::value;
-            C Cs = x[0], Sn = CT<C>::mk(0, 0);
-            static_for<1, H + 1>([&](auto jc) {
-                constexpr int k = decltype(jc)::value;
-                constexpr CxCis w = cx_cis((long)k * kap, NK);
-                Cs.x = fma(p[k].x, (R)w.c, Cs.x);
-                Cs.y = fma(p[k].y, (R)w.c, Cs.y);
-                Sn.x = fma(q[k].x, (R)w.s, Sn.x);
-                Sn.y = fma(q[k].y, (R)w.s, Sn.y);
-            });
-            if constexpr (EVEN) {
-                constexpr R e = (kap & 1) ? (R)-1 : (R)1;
-                Cs.x = fma(e, xh.x, Cs.x);
-                Cs.y = fma(e, xh.y, Cs.y);
-            }
-            X[(size_t)kap * M + m] = CT<C>::mk(Cs.x - sgn * Sn.y, Cs.y + sgn * Sn.x);
-            X[(size_t)(NK - kap) * M + m] = CT<C>::mk(Cs.x + sgn * Sn.y, Cs.y - sgn * Sn.x);
-        });
-        if constexpr (EVEN && NK > 1) {  // kappa = NK/2: cos(pi k) = (-1)^k, sin = 0
-            C Cs = x[0];
-#pragma unroll
-            for (int k = 1; k <= H; ++k) {
-                const R e = (k & 1) ? (R)-1 : (R)1;
-                Cs.x = fma(e, p[k].x, Cs.x);
-                Cs.y = fma(e, p[k].y, Cs.y);
-            }
-            constexpr R e = ((NK / 2) & 1) ? (R)-1 : (R)1;
-            X[(size_t)(NK / 2) * M + m] = CT<C>::mk(fma(e, xh.x, Cs.x), fma(e, xh.y, Cs.y));
-        }
+        kz_dft<C, NK>(x, inverse, [&](int kap, C v) { X[(size_t)kap * M + m] = v; });
     }
 }
 

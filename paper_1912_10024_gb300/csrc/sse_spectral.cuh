@@ -142,12 +142,13 @@ struct CX<float> {
     using C = float2;
 };
 
-// tw[m] = exp(-2 pi i m / L)
-__global__ void twiddle_kernel(int L, double2* __restrict__ tw) {
+// tw[m] = exp(-2 pi i m / L), in the precision of the transforms
+template <class C>
+__global__ void twiddle_kernel(int L, C* __restrict__ tw) {
     for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < L; m += gridDim.x * blockDim.x) {
         double s, c;
         sincospi(2.0 * (double)m / (double)L, &s, &c);
-        tw[m] = make_double2(c, -s);
+        tw[m] = CT<C>::mk(c, -s);
     }
 }
 
@@ -351,7 +352,8 @@ struct StoreSigmaT {  // S[k][E][a_begin*nel + col] = conj(v) * inv in FP64, E <
 using StoreSigma = StoreSigmaT<double2>;
 
 template <class Load, class Store, int CC>
-__global__ void __launch_bounds__(kFftThreads) fft_e_kernel(FftPlan p, const double2* __restrict__ tw_g, Load ld,
+__global__ void __launch_bounds__(kFftThreads) fft_e_kernel(FftPlan p,
+                                                            const typename Load::C* __restrict__ tw_g, Load ld,
                                                             Store sv, size_t ncols) {
     using C = typename Load::C;
     constexpr int lgC = CC == 1 ? 0 : CC == 2 ? 1 : CC == 4 ? 2 : CC == 8 ? 3 : 4;
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(kFftThreads) fft_e_kernel(FftPlan p, const dou
     C* tw = b1 + p.L * CC;
     const size_t col0 = (size_t)blockIdx.x * CC;
     const int batch = blockIdx.y;
-    for (int m = threadIdx.x; m < p.L; m += blockDim.x) tw[m] = CT<C>::mk(tw_g[m].x, tw_g[m].y);
+    for (int m = threadIdx.x; m < p.L; m += blockDim.x) tw[m] = tw_g[m];
     const int n = p.L * CC;
     for (int base = threadIdx.x; base < n; base += kFftLoadBatch * blockDim.x) {
         C v[kFftLoadBatch];
@@ -567,7 +569,7 @@ inline unsigned grid_for(size_t work, int threads) {
 }
 
 template <int CC, class Load, class Store>
-cudaError_t launch_fft_c(const char* name, const FftPlan& p, const double2* tw, Load ld, Store sv, size_t ncols,
+cudaError_t launch_fft_c(const char* name, const FftPlan& p, const typename Load::C* tw, Load ld, Store sv, size_t ncols,
                          int batches, cudaStream_t st) {
     cudaError_t e =
         cudaFuncSetAttribute(fft_e_kernel<Load, Store, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
@@ -581,7 +583,7 @@ cudaError_t launch_fft_c(const char* name, const FftPlan& p, const double2* tw, 
 }
 
 template <class Load, class Store>
-cudaError_t launch_fft(const char* name, const FftPlan& p, const double2* tw, Load ld, Store sv, size_t ncols,
+cudaError_t launch_fft(const char* name, const FftPlan& p, const typename Load::C* tw, Load ld, Store sv, size_t ncols,
                        int batches, cudaStream_t st) {
     switch (p.C) {
         case 16: return launch_fft_c<16>(name, p, tw, ld, sv, ncols, batches, st);

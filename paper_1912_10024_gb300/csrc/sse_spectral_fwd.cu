@@ -207,7 +207,7 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
     const SpecLayout lay = spec_layout(d, sizeof(C));
     if (ws_bytes < lay.total) return cudaErrorInvalidValue;
     unsigned char* base = static_cast<unsigned char*>(ws);
-    double2* tw = reinterpret_cast<double2*>(base + lay.off_tw);
+    C* tw = reinterpret_cast<C*>(base + lay.off_tw);
     C* Gh = reinterpret_cast<C*>(base + lay.off_G);
     C* Kh = reinterpret_cast<C*>(base + lay.off_K);
     C* Sh = reinterpret_cast<C*>(base + lay.off_S);

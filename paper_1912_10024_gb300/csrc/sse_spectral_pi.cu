@@ -525,7 +525,7 @@ cudaError_t spectral_pi_t(const sse_dims& d, const int32_t* nbr, const double2* 
     const PiLayout lay = pi_layout(d, sizeof(C));
     if (ws_bytes < lay.total) return cudaErrorInvalidValue;
     unsigned char* base = static_cast<unsigned char*>(ws);
-    double2* tw = reinterpret_cast<double2*>(base + lay.off_tw);
+    C* tw = reinterpret_cast<C*>(base + lay.off_tw);
     C* Gh[2] = {reinterpret_cast<C*>(base + lay.off_G[0]), reinterpret_cast<C*>(base + lay.off_G[1])};
     C* Ch[2] = {reinterpret_cast<C*>(base + lay.off_C[0]), reinterpret_cast<C*>(base + lay.off_C[1])};
     const int L = lay.L;
