@@ -3,6 +3,7 @@
 // drivers (device buffers, and the pipelined variant behind the host-buffer entry point). Mode F16X3_FFT runs the
 // same FP32 transforms with the block products of sse_spectral_tc.cu on the tensor cores.
 #include "sse_prod32.cuh"
+#include "sse_tri.cuh"
 
 namespace sse {
 namespace {
@@ -236,6 +237,13 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
+    // anti-Hermitian blocks: transforms of the upper triangle's columns (sse_tri.cuh). The triangle of G^ sits in S^'s
+    // region until the products write there, that of S^ in G^'s after them.
+    const TriMap tri = make_tri_map(d.Norb);
+    const bool use_tri = half && tri_applies(d, L, (size_t)d.Nkz * L * scols);
+    const size_t tg = (size_t)d.NA * tri.nt, ts = nA * tri.nt;  // columns
+    C* Gc = Sh;
+    C* Sc = Gh;
     const ProdCfg pc = make_prod_cfg(d, fm.count, (int)sizeof(T));
     constexpr bool tiled = sizeof(T) == 4;  // FP32: register-tiled kernel
     if constexpr (!tiled)
@@ -251,19 +259,21 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
         if (e != cudaSuccess) return e;
         if ((e = launch_dft_k("dft_kz_kernel(K)", Kh, d.Nkz, d.Nqz, (size_t)L * kcols, 0, st)) != cudaSuccess) return e;
         // 2. G^t -> G^ (E-transform per kz slice as the slices arrive, then the kz DFT)
-        if (pipe) {
-            for (int k = 0; k < d.Nkz; ++k) {
-                if ((e = cudaStreamWaitEvent(st, pipe->g[t][k], 0)) != cudaSuccess) return e;
-                e = launch_fft32("fft_e_kernel(G)", plan, tw, LoadGT<C>{p.G[t] + (size_t)k * d.NE * gcols, d.NE, gcols},
-                               StoreSpecT<C>{Gh + (size_t)k * L * gcols, L, gcols, L}, gcols, 1, st);
-                if (e != cudaSuccess) return e;
-            }
-        } else {
-            e = launch_fft32("fft_e_kernel(G)", plan, tw, LoadGT<C>{p.G[t], d.NE, gcols},
-                           StoreSpecT<C>{Gh, L, gcols, L}, gcols, d.Nkz, st);
+        const int gslices = pipe ? d.Nkz : 1, gper = pipe ? 1 : d.Nkz;
+        for (int k = 0; k < gslices; ++k) {
+            if (pipe && (e = cudaStreamWaitEvent(st, pipe->g[t][k], 0)) != cudaSuccess) return e;
+            const double2* Gk = p.G[t] + (size_t)k * d.NE * gcols;
+            if (use_tri)
+                e = launch_fft32("fft_e_kernel(G)", plan, tw, LoadGTri<C>{Gk, d.NE, gcols, tri},
+                                 StoreSpecT<C>{Gc + (size_t)k * L * tg, L, tg, L}, tg, gper, st);
+            else
+                e = launch_fft32("fft_e_kernel(G)", plan, tw, LoadGT<C>{Gk, d.NE, gcols},
+                                 StoreSpecT<C>{Gh + (size_t)k * L * gcols, L, gcols, L}, gcols, gper, st);
             if (e != cudaSuccess) return e;
         }
-        if ((e = launch_dft_k("dft_kz_kernel(G)", Gh, d.Nkz, d.Nkz, (size_t)L * gcols, 0, st)) != cudaSuccess) return e;
+        e = use_tri ? launch_kz_expand("dft_kz_expand_kernel(G)", Gc, Gh, tri, d.Nkz, L, tg, false, st)
+                    : launch_dft_k("dft_kz_kernel(G)", Gh, d.Nkz, d.Nkz, (size_t)L * gcols, 0, st);
+        if (e != cudaSuccess) return e;
         // 3. block products (one frequency of each (f, -f) pair with anti-Hermitian inputs, then the mirror)
         if (tc) {
             e = spectral_prod_tc(d, fm, p.nbr, p.dH, reinterpret_cast<const float2*>(Gh),
@@ -280,41 +290,37 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
                           pc, d, fm, p.nbr, p.dH, Gh, Kh, Sh, p.scale, status));
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (half) {
+        if (half && !use_tri) {
             SSE_TIMED("mirror_sigma_kernel", st,
                       mirror_sigma_kernel<<<grid_for(fm.count * nA * nel, 256), 256, 0, st>>>(fm, nA, d.Norb, Sh));
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
         // 4. inverse transforms into Sigma^t
-        if ((e = launch_dft_k("dft_kz_kernel(S)", Sh, d.Nkz, d.Nkz, (size_t)L * scols, 1, st)) != cudaSuccess) return e;
+        e = use_tri ? launch_kz_compress("dft_kz_compress_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st)
+                    : launch_dft_k("dft_kz_kernel(S)", Sh, d.Nkz, d.Nkz, (size_t)L * scols, 1, st);
+        if (e != cudaSuccess) return e;
         const double inv = 1.0 / ((double)d.Nkz * (double)L);
         const bool sym = (p.flags & SSE_FLAG_SYMMETRIZE) != 0;
-        if (pipe) {  // slice by slice, each handed to its download as soon as it is written
-            sse_dims dk = d;
-            dk.Nkz = 1;
-            for (int k = 0; k < d.Nkz; ++k) {
-                double2* Sk = S[t] + (size_t)k * d.NE * d.NA * nel;
+        // with `pipe` slice by slice, each handed to its download as soon as it is written
+        const int sslices = pipe ? d.Nkz : 1, sper = pipe ? 1 : d.Nkz;
+        sse_dims dk = d;
+        dk.Nkz = sper;
+        for (int k = 0; k < sslices; ++k) {
+            double2* Sk = S[t] + (size_t)k * d.NE * d.NA * nel;
+            if (use_tri)
+                e = launch_fft32("fft_e_kernel(S)", plan, tw, LoadSpecConjT<C>{Sc + (size_t)k * L * ts, L, ts},
+                                 StoreSigmaTri<C>{Sk, d.NE, gcols, (size_t)d.a_begin * nel, inv, d.NE, sym ? 1 : 0, tri},
+                                 ts, sper, st);
+            else
                 e = launch_fft32("fft_e_kernel(S)", plan, tw, LoadSpecConjT<C>{Sh + (size_t)k * L * scols, L, scols},
-                               StoreSigmaT<C>{Sk, d.NE, (size_t)d.NA * nel, (size_t)d.a_begin * nel, inv, d.NE},
-                               scols, 1, st);
-                if (e != cudaSuccess) return e;
-                if (sym) {
-                    SSE_TIMED("symmetrize_kernel", st,
-                              symmetrize_kernel<<<grid_for((size_t)d.NE * nA * nel, 256), 256, 0, st>>>(dk, Sk));
-                    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-                }
-                if ((e = cudaEventRecord(pipe->s[t][k], st)) != cudaSuccess) return e;
-            }
-        } else {
-            e = launch_fft32("fft_e_kernel(S)", plan, tw, LoadSpecConjT<C>{Sh, L, scols},
-                           StoreSigmaT<C>{S[t], d.NE, (size_t)d.NA * nel, (size_t)d.a_begin * nel, inv, d.NE}, scols,
-                           d.Nkz, st);
+                                 StoreSigmaT<C>{Sk, d.NE, gcols, (size_t)d.a_begin * nel, inv, d.NE}, scols, sper, st);
             if (e != cudaSuccess) return e;
-            if (sym) {
+            if (sym && !use_tri) {
                 SSE_TIMED("symmetrize_kernel", st,
-                          symmetrize_kernel<<<grid_for((size_t)d.Nkz * d.NE * nA * nel, 256), 256, 0, st>>>(d, S[t]));
+                          symmetrize_kernel<<<grid_for((size_t)sper * d.NE * nA * nel, 256), 256, 0, st>>>(dk, Sk));
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
             }
+            if (pipe && (e = cudaEventRecord(pipe->s[t][k], st)) != cudaSuccess) return e;
         }
     }
     return cudaSuccess;

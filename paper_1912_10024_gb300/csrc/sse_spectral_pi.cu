@@ -1,6 +1,7 @@
 // Pi of Eq. (4) through the transforms: the per-frequency half products and traces in FP64 (spec_pi_kernel) and
 // FP32 (spec_pi32_kernel), the store of the inverse transform, the 3x3 symmetrisation and the driver.
 #include "sse_prod32.cuh"
+#include "sse_tri.cuh"
 
 namespace sse {
 namespace {
@@ -537,14 +538,27 @@ cudaError_t spectral_pi_t(const sse_dims& d, const int32_t* nbr, const double2* 
     SSE_TIMED("twiddle_kernel", st, twiddle_kernel<<<grid_for(L, 256), 256, 0, st>>>(L, tw));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const double2* G[2] = {G_less, G_greater};
+    const bool half = (flags & SSE_FLAG_ANTIHERMITIAN) != 0;
+    const FreqMap fm = make_freq_map(d.Nkz, L, half);
+    // anti-Hermitian blocks: transforms of the upper triangle's columns (sse_tri.cuh), one type at a time in the region of
+    // both C^ spectra, which the products write later
+    const TriMap tri = make_tri_map(d.Norb);
+    const size_t tg = (size_t)d.NA * tri.nt;
+    const bool use_tri = half && tri_applies(d, L, (lay.total - lay.off_C[0]) / sizeof(C));
     for (int t = 0; t < 2; ++t) {
+        if (use_tri) {
+            e = launch_fft32("fft_e_kernel(G)", plan, tw, LoadGTri<C>{G[t], d.NE, gcols, tri},
+                             StoreSpecT<C>{Ch[0], L, tg, L}, tg, d.Nkz, st);
+            if (e != cudaSuccess) return e;
+            e = launch_kz_expand("dft_kz_expand_kernel(G)", Ch[0], Gh[t], tri, d.Nkz, L, tg, true, st);
+            if (e != cudaSuccess) return e;
+            continue;
+        }
         e = launch_fft32("fft_e_kernel(G)", plan, tw, LoadGT<C>{G[t], d.NE, gcols}, StoreSpecT<C>{Gh[t], L, gcols, L},
                        gcols, d.Nkz, st);
         if (e != cudaSuccess) return e;
         if ((e = launch_dft_k("dft_kz_kernel(G)", Gh[t], d.Nkz, d.Nkz, (size_t)L * gcols, 0, st)) != cudaSuccess) return e;
     }
-    const bool half = (flags & SSE_FLAG_ANTIHERMITIAN) != 0;
-    const FreqMap fm = make_freq_map(d.Nkz, L, half);
     if (half && (flags & SSE_FLAG_CHECK))
         for (int t = 0; t < 2; ++t) {
             SSE_TIMED("check_antiherm_kernel", st,
