@@ -128,23 +128,43 @@ __global__ void spec_prod_kernel(ProdCfg c, sse_dims d, FreqMap fm, const int32_
     }
 }
 
-// (S - S^H)/2 on the blocks of atoms in range
-__global__ void symmetrize_kernel(sse_dims d, double2* __restrict__ S) {
-    const int Norb = d.Norb, nel = Norb * Norb;
+// (S - S^H)/2 on the blocks of atoms in range. A CTA takes about 1024 elements of whole blocks through shared memory, so
+// that the accesses are contiguous although every element meets its transposed one, and divides 64-bit indices once per
+// block. NA = 90, Norb = 7, NE = 301, Nkz = 4, both types: 131 -> 96 us (340 MB, 50 us; the FP64 operations 35 us). Forming
+// each pair of elements once halves those but adds a pass over shared memory: 120 us.
+constexpr int kSymElems = 1024, kSymThreads = 256;
+
+__global__ void __launch_bounds__(kSymThreads) symmetrize_kernel(sse_dims d, double2* __restrict__ S) {
+    __shared__ double2 tile[kSymElems];
+    __shared__ double2* base[kSymElems];
+    const int Norb = d.Norb, nel = Norb * Norb, per = kSymElems / nel;  // nel <= 256
     const size_t nA = (size_t)(d.a_end - d.a_begin);
     const size_t nblk = (size_t)d.Nkz * d.NE * nA;
-    const size_t total = nblk * nel;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int e = (int)(i % nel);
-        const size_t blk = i / nel;
-        const int m = e / Norb, n = e - m * Norb;
-        if (n < m) continue;
-        const size_t ke = blk / nA, la = blk - ke * nA;
-        double2* B = S + (ke * d.NA + d.a_begin + la) * nel;
-        const double2 x = B[m * Norb + n], y = B[n * Norb + m];
-        B[m * Norb + n] = make_double2(0.5 * (x.x - y.x), 0.5 * (x.y + y.y));
-        if (m != n) B[n * Norb + m] = make_double2(0.5 * (y.x - x.x), 0.5 * (y.y + x.y));
+    for (size_t b0 = (size_t)blockIdx.x * per; b0 < nblk; b0 += (size_t)gridDim.x * per) {
+        const int nb = (int)min((size_t)per, nblk - b0);
+        for (int i = threadIdx.x; i < nb; i += kSymThreads) {
+            const size_t ke = (b0 + i) / nA, la = b0 + i - ke * nA;
+            base[i] = S + (ke * d.NA + d.a_begin + la) * nel;
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < nb * nel; i += kSymThreads) {
+            const int blk = i / nel;
+            tile[i] = base[blk][i - blk * nel];
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < nb * nel; i += kSymThreads) {
+            const int blk = i / nel, e = i - blk * nel, m = e / Norb, n = e - m * Norb;
+            const double2 x = tile[i], y = tile[blk * nel + n * Norb + m];
+            base[blk][e] = make_double2(0.5 * (x.x - y.x), 0.5 * (x.y + y.y));
+        }
+        __syncthreads();  // tile and base are rewritten
     }
+}
+
+inline unsigned symmetrize_grid(const sse_dims& d, int Nkz) {
+    const size_t nblk = (size_t)Nkz * d.NE * (size_t)(d.a_end - d.a_begin);
+    const size_t per = kSymElems / (d.Norb * d.Norb), g = (nblk + per - 1) / per;
+    return (unsigned)(g < 1 ? 1 : g > 0x7fffffff ? 0x7fffffff : g);
 }
 
 struct SpecLayout {
@@ -317,7 +337,7 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
             if (e != cudaSuccess) return e;
             if (sym && !use_tri) {
                 SSE_TIMED("symmetrize_kernel", st,
-                          symmetrize_kernel<<<grid_for((size_t)sper * d.NE * nA * nel, 256), 256, 0, st>>>(dk, Sk));
+                          symmetrize_kernel<<<symmetrize_grid(d, sper), kSymThreads, 0, st>>>(dk, Sk));
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
             }
             if (pipe && (e = cudaEventRecord(pipe->s[t][k], st)) != cudaSuccess) return e;
