@@ -99,8 +99,9 @@ typedef struct sse_dims {
  *            power-of-two normalisation, wider accumulation). Frequencies stack into the
  *            rows of two GEMMs per bond whose second operand, dH, is shared by every
  *            frequency; each operand is scaled by a power of two and split into FP16
- *            hi + lo, and hi*hi + hi*lo + lo*hi accumulate in FP32. Error (normwise)
- *            a few 1e-7, tested to 2e-6. sse_sigma_fwd and sse_sigma_fwd_host only;
+ *            hi + lo, and hi*hi + hi*lo + lo*hi accumulate in FP32. Where the FP32
+ *            products of FP32_FFT are faster (Norb < 9 or NB < 3) they are used instead
+ *            (no less precise). Error (normwise) a few 1e-7, tested to 2e-6. sse_sigma_fwd and sse_sigma_fwd_host only;
  *            FP32_FFT's workspace; needs Norb <= 10 and NB <= 4 besides the transform
  *            limits (else SSE_ERR_UNSUPPORTED before any device work). */
 typedef enum sse_mode {

@@ -430,6 +430,7 @@ __device__ __forceinline__ size_t freq_neg(const FreqMap& m, size_t f) {
 // FP32 spectra G^ [Nkz*L][NA][Norb^2] and K^ [Nkz*L][nA][NB][9] into S^ [Nkz*L][nA][Norb^2] (frequencies of `fm`).
 // Limits (host-only): Norb <= 10, NB <= 4.
 bool spectral_prod_tc_supported(const sse_dims& d);
+bool spectral_prod_tc_pays(const sse_dims& d);  // where the FP32 products of sse_prod32.cuh are slower
 cudaError_t spectral_prod_tc(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, const double2* dH,
                              const float2* Gh, const float2* Kh, float2* Sh, double scale, unsigned* status,
                              cudaStream_t st);

@@ -222,7 +222,7 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
     // can start; without it every transform is one launch over all slices.
     using C = typename CX<T>::C;
     const sse_dims& d = p.d;
-    // tc: the FP32 transforms with the block products on the tensor cores (mode F16X3_FFT)
+    // tc: mode F16X3_FFT, the FP32 transforms with the block products on the tensor cores where those are faster
     if (tc && sizeof(T) != 4) return cudaErrorNotSupported;
     if (!(tc ? spectral_fwd_tc_supported(d) : spectral_fwd_supported(d, sizeof(T) == 4))) return cudaErrorNotSupported;
     const SpecLayout lay = spec_layout(d, sizeof(C));
@@ -295,7 +295,7 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
                     : launch_dft_k("dft_kz_kernel(G)", Gh, d.Nkz, d.Nkz, (size_t)L * gcols, 0, st);
         if (e != cudaSuccess) return e;
         // 3. block products (one frequency of each (f, -f) pair with anti-Hermitian inputs, then the mirror)
-        if (tc) {
+        if (tc && spectral_prod_tc_pays(d)) {
             e = spectral_prod_tc(d, fm, p.nbr, p.dH, reinterpret_cast<const float2*>(Gh),
                                  reinterpret_cast<const float2*>(Kh), reinterpret_cast<float2*>(Sh), p.scale, status,
                                  st);

@@ -746,18 +746,17 @@ bool spectral_prod_tc_supported(const sse_dims& d) {
     }
 }
 
+// The tensor cores pay for large blocks with several bonds only: a tile of 128 rows costs about the same for every Norb
+// (the work around its GEMMs is a chain of latencies), and it holds fewer frequencies of few bonds. Products of both types,
+// tensor cores / FP32 CUDA cores, NA = 256, NE = 256, Nkz = 5: NB = 4: Norb 4 1169 / 393 us, 6 1783 / 897, 7 2280 / 2027, 8
+// 2361 / 1841, 9 3210 / 3704, 10 3275 / 3395; NB = 3: 8 1805 / 1395, 9 2501 / 2795, 10 2534 / 2561; NB = 1: 9 1071 / 989,
+// 10 1067 / 900. The FP32 products keep more bits than the split FP16 operands.
+bool spectral_prod_tc_pays(const sse_dims& d) { return d.Norb >= 9 && d.NB >= 3; }
+
 cudaError_t spectral_prod_tc(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, const double2* dH,
                              const float2* Gh, const float2* Kh, float2* Sh, double scale, unsigned* status,
                              cudaStream_t st) {
     switch (d.Norb) {
-        case 1: return launch_tc<1>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
-        case 2: return launch_tc<2>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
-        case 3: return launch_tc<3>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
-        case 4: return launch_tc<4>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
-        case 5: return launch_tc<5>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
-        case 6: return launch_tc<6>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
-        case 7: return launch_tc<7>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
-        case 8: return launch_tc<8>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
         case 9: return launch_tc<9>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
         case 10: return launch_tc<10>(d, fm, nbr, dH, Gh, Kh, Sh, scale, status, st);
         default: return cudaErrorNotSupported;
