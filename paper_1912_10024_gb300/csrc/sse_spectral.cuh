@@ -305,9 +305,10 @@ struct LoadLagT {
     int Nw, L;
     size_t rowlen, col0;
     __device__ C operator()(int q, int r, size_t col) const {
-        double2 v = make_double2(0.0, 0.0);
-        if (r >= 1 && r <= Nw) v = Dt[((size_t)q * Nw + (r - 1)) * rowlen + col0 + col];
-        else if (r >= L - Nw) v = Dtb[((size_t)q * Nw + (L - 1 - r)) * rowlen + col0 + col];
+        const bool up = r >= 1 && r <= Nw, down = r >= L - Nw;
+        if (!up && !down) return CT<C>::mk(0, 0);  // most rows: no conversion of zeros: FinFET, both types, FP32
+        // transforms 1.57 -> 0.93 ms
+        const double2 v = (up ? Dt : Dtb)[((size_t)q * Nw + (up ? r - 1 : L - 1 - r)) * rowlen + col0 + col];
         return CT<C>::mk(v.x, v.y);
     }
 };

@@ -262,6 +262,11 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
     const TriMap tri = make_tri_map(d.Norb);
     const bool use_tri = half && tri_applies(d, L, (size_t)d.Nkz * L * scols);
     const size_t tg = (size_t)d.NA * tri.nt, ts = nA * tri.nt;  // columns
+    // the same for the 3 x 3 blocks of the lag kernel, whose triangle comes before that of G^ in S^'s region
+    const TriMap tri3 = make_tri_map(3);
+    const size_t tk = nA * d.NB * tri3.nt;
+    const bool use_tri3 = use_tri && tk <= scols && tk <= 0x7fffffffu;
+    C* Kc = Sh;
     C* Gc = Sh;
     C* Sc = Gh;
     const ProdCfg pc = make_prod_cfg(d, fm.count, (int)sizeof(T));
@@ -274,10 +279,20 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
     if (pipe && (e = cudaStreamWaitEvent(st, pipe->inputs, 0)) != cudaSuccess) return e;
     for (int t = 0; t < 2; ++t) {
         // 1. lag kernel -> K^ (needs only D; with `pipe` it runs while G^t is still arriving)
-        LoadLagT<C> ll{p.D[t], p.D[1 - t], d.Nw, L, (size_t)d.NA * d.NB * 9, (size_t)d.a_begin * d.NB * 9};
-        e = launch_fft32("fft_e_kernel(K)", plan, tw, ll, StoreSpecT<C>{Kh, L, kcols, L}, kcols, d.Nqz, st);
+        const size_t rowlen = (size_t)d.NA * d.NB * 9, kcol0 = (size_t)d.a_begin * d.NB * 9;
+        if (use_tri3) {
+            e = launch_fft32("fft_e_kernel(K)", plan, tw,
+                             LoadLagTri<C>{p.D[t], p.D[1 - t], d.Nw, L, rowlen, kcol0, tri3},
+                             StoreSpecT<C>{Kc, L, tk, L}, tk, d.Nqz, st);
+            if (e != cudaSuccess) return e;
+            e = launch_kz_expand("dft_kz_expand_kernel(K)", Kc, Kh, tri3, d.Nkz, d.Nqz, L, tk, false, st);
+        } else {
+            e = launch_fft32("fft_e_kernel(K)", plan, tw, LoadLagT<C>{p.D[t], p.D[1 - t], d.Nw, L, rowlen, kcol0},
+                             StoreSpecT<C>{Kh, L, kcols, L}, kcols, d.Nqz, st);
+            if (e != cudaSuccess) return e;
+            e = launch_dft_k("dft_kz_kernel(K)", Kh, d.Nkz, d.Nqz, (size_t)L * kcols, 0, st);
+        }
         if (e != cudaSuccess) return e;
-        if ((e = launch_dft_k("dft_kz_kernel(K)", Kh, d.Nkz, d.Nqz, (size_t)L * kcols, 0, st)) != cudaSuccess) return e;
         // 2. G^t -> G^ (E-transform per kz slice as the slices arrive, then the kz DFT)
         const int gslices = pipe ? d.Nkz : 1, gper = pipe ? 1 : d.Nkz;
         for (int k = 0; k < gslices; ++k) {
@@ -291,7 +306,7 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
                                  StoreSpecT<C>{Gh + (size_t)k * L * gcols, L, gcols, L}, gcols, gper, st);
             if (e != cudaSuccess) return e;
         }
-        e = use_tri ? launch_kz_expand("dft_kz_expand_kernel(G)", Gc, Gh, tri, d.Nkz, L, tg, false, st)
+        e = use_tri ? launch_kz_expand("dft_kz_expand_kernel(G)", Gc, Gh, tri, d.Nkz, d.Nkz, L, tg, false, st)
                     : launch_dft_k("dft_kz_kernel(G)", Gh, d.Nkz, d.Nkz, (size_t)L * gcols, 0, st);
         if (e != cudaSuccess) return e;
         // 3. block products (one frequency of each (f, -f) pair with anti-Hermitian inputs, then the mirror)

@@ -550,7 +550,7 @@ cudaError_t spectral_pi_t(const sse_dims& d, const int32_t* nbr, const double2* 
             e = launch_fft32("fft_e_kernel(G)", plan, tw, LoadGTri<C>{G[t], d.NE, gcols, tri},
                              StoreSpecT<C>{Ch[0], L, tg, L}, tg, d.Nkz, st);
             if (e != cudaSuccess) return e;
-            e = launch_kz_expand("dft_kz_expand_kernel(G)", Ch[0], Gh[t], tri, d.Nkz, L, tg, true, st);
+            e = launch_kz_expand("dft_kz_expand_kernel(G)", Ch[0], Gh[t], tri, d.Nkz, d.Nkz, L, tg, true, st);
             if (e != cudaSuccess) return e;
             continue;
         }

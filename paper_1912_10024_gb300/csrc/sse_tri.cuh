@@ -4,8 +4,9 @@
 // computed half of the frequencies (and of the other half where Pi needs it), and after the products the inverse kz DFT
 // reads that half and writes the triangle's columns for every frequency. 0.55 of the E-transforms at Norb = 10, half of
 // the kz passes, no mirror pass, no separate symmetrisation.
-// FinFET in FP64 (the transforms are bound by the FP64 pipe): E-transforms of G and S 102 -> 58 ms, their kz passes 31 -> 17
-// ms, mirror 3.6 -> 0: the step 830 -> 768 ms.
+// The 3 x 3 blocks of the lag kernel
+// are taken the same way (six columns of nine). FinFET in FP64 (the transforms are bound by the FP64 pipe): E-transforms
+// of G and S 102 -> 58 ms, of K 17.6 -> 11.8; kz passes 36 -> 21 ms, mirror 3.6 -> 0: the call 830 -> 761 ms.
 #pragma once
 
 #include "sse_spectral.cuh"
@@ -47,6 +48,26 @@ struct LoadGTri {
     }
 };
 
+// lag kernel of one qz slice (LoadLagT) for the triangle of its 3 x 3 blocks: row w + 1 <- D^t(q, w), row L - (w + 1) <-
+// D^t'(q, w), else zero
+template <class CC>
+struct LoadLagTri {
+    using C = CC;
+    const double2* Dt;
+    const double2* Dtb;
+    int Nw, L;
+    size_t rowlen, col0;
+    TriMap t;
+    __device__ C operator()(int q, int r, size_t col) const {
+        const bool up = r >= 1 && r <= Nw, down = r >= L - Nw;
+        if (!up && !down) return CT<C>::mk(0, 0);
+        const unsigned b = (unsigned)col / (unsigned)t.nt;
+        const size_t at = (size_t)b * t.nel + t.at[(unsigned)col - b * t.nt];
+        const double2 v = (up ? Dt : Dtb)[((size_t)q * Nw + (up ? r - 1 : L - 1 - r)) * rowlen + col0 + at];
+        return CT<C>::mk(v.x, v.y);
+    }
+};
+
 // S[k][E][a_begin * nel + atom * nel + mn] = conj(v) * inv and its partner -conj at nm, E < NE; with sym the diagonal's
 // real part (rounding) is cleared, as (S - S^H) / 2 does
 template <class C>
@@ -76,11 +97,11 @@ struct StoreSigmaTri {
 __device__ __forceinline__ double2 cnegconj(double2 a) { return make_double2(-a.x, a.y); }
 __device__ __forceinline__ float2 cnegconj(float2 a) { return make_float2(-a.x, a.y); }
 
-// forward kz DFT of the triangle's columns X[k][eps][atom][i] into full blocks G[kappa][eps][atom][mn] for eps <= L / 2,
+// forward kz DFT of the triangle's columns X[k < n_in][eps][block][i] into full blocks G[kappa][eps][block][mn] for eps <= L / 2,
 // and for every eps with `both`. A thread takes the rows eps and L - eps of one column.
 template <class C, int NK>
-__global__ void __launch_bounds__(256) dft_kz_expand_kernel(const C* __restrict__ X, C* __restrict__ G, TriMap t, int L,
-                                                            unsigned ncols, int both) {
+__global__ void __launch_bounds__(256) dft_kz_expand_kernel(const C* __restrict__ X, C* __restrict__ G, TriMap t, int n_in,
+                                                            int L, unsigned ncols, int both) {
     const size_t total = (size_t)(L / 2 + 1) * ncols;
     const size_t gcols = (size_t)(ncols / t.nt) * t.nel;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
@@ -89,7 +110,7 @@ __global__ void __launch_bounds__(256) dft_kz_expand_kernel(const C* __restrict_
         const int at = t.at[k0], tr = t.tr[k0];
         C x[NK];
 #pragma unroll
-        for (int k = 0; k < NK; ++k) x[k] = X[((size_t)k * L + e) * ncols + col];
+        for (int k = 0; k < NK; ++k) x[k] = k < n_in ? X[((size_t)k * L + e) * ncols + col] : CT<C>::mk(0, 0);
         C* g = G + (size_t)e * gcols + (size_t)a * t.nel;    // row eps
         C* gm = G + (size_t)em * gcols + (size_t)a * t.nel;  // row -eps
         const size_t slab = (size_t)L * gcols;
@@ -101,7 +122,7 @@ __global__ void __launch_bounds__(256) dft_kz_expand_kernel(const C* __restrict_
         });
         if (self || diag) continue;
 #pragma unroll
-        for (int k = 0; k < NK; ++k) x[k] = X[((size_t)k * L + em) * ncols + col];
+        for (int k = 0; k < NK; ++k) x[k] = k < n_in ? X[((size_t)k * L + em) * ncols + col] : CT<C>::mk(0, 0);
         kz_dft<C, NK>(x, 0, [&](int kap, C v) {
             const int km = kap == 0 ? 0 : NK - kap;
             g[km * slab + tr] = cnegconj(v);
@@ -161,12 +182,12 @@ cudaError_t tri_with_nk(int nk, F&& f) {
 }
 
 template <class C>
-cudaError_t launch_kz_expand(const char* name, const C* X, C* G, const TriMap& t, int Nk, int L, size_t ncols, bool both,
-                             cudaStream_t st) {
+cudaError_t launch_kz_expand(const char* name, const C* X, C* G, const TriMap& t, int Nk, int n_in, int L, size_t ncols,
+                             bool both, cudaStream_t st) {
     return tri_with_nk(Nk, [&](auto nk) {
         SSE_TIMED(name, st,
                   dft_kz_expand_kernel<C, decltype(nk)::value>
-                  <<<grid_for((size_t)(L / 2 + 1) * ncols, 256), 256, 0, st>>>(X, G, t, L, (unsigned)ncols, both ? 1 : 0));
+                  <<<grid_for((size_t)(L / 2 + 1) * ncols, 256), 256, 0, st>>>(X, G, t, n_in, L, (unsigned)ncols, both ? 1 : 0));
         return cudaGetLastError();
     });
 }
