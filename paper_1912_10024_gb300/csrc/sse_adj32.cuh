@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(AdjShape<NP>::THREADS, AdjShape<NP>::CTAS) spe
                             w[f][r] = lds4(W + (fs + f * S::FG) * XS + ((2 * mp + r) * NP + l0) * 2);
 #pragma unroll
                     for (int dl = 0; dl < 2; ++dl) {
+                        if (ODD && l0 + dl >= N) continue;  // the padding column of an odd block
                         float4 g[NF];  // G[l][n] of the two columns
 #pragma unroll
                         for (int f = 0; f < NF; ++f)
@@ -322,8 +323,8 @@ __global__ void __launch_bounds__(AdjShape<NP>::THREADS, AdjShape<NP>::CTAS) spe
                 const float* scal = part == 0 ? G + k0 * NP * 2 : W + k0 * 2;
                 const int sl = part == 0 ? 2 : NP * 2, sk = part == 0 ? NP * 2 : 2;
 #pragma unroll 1
-                for (int u = gr >> 1; u < F * NP; u += S::GP) {
-                    const int f = u / NP, l = u - f * NP;
+                for (int u = gr >> 1; u < F * N; u += S::GP) {
+                    const int f = u / N, l = u - f * N;
                     float2 z[RH];
 #pragma unroll
                     for (int k = 0; k < RH; ++k) z[k] = ld2(scal + f * XS + l * sl + k * sk);

@@ -74,11 +74,12 @@ struct TileShape {
     static constexpr int RH = NP / 2;               // rows per thread
     static constexpr int CP = NP / 2;               // column pairs
     static constexpr int TPF = 2 * CP;              // threads per frequency set
-    static constexpr int NF = NP <= 8 ? 2 : 1;      // frequencies per thread: two while their tiles fit in registers
+    static constexpr int NF = NP <= 6 ? 2 : 1;      // frequencies per thread: two while their tiles fit in registers
     // CTAs per SM that the registers (P 12 Np NF / 2, acc 2 Np NF, operands) leave room for without spills. Measured at
     // Norb = 10: NF = 1 with three CTAs 36.6 ms per FinFET step, NF = 2 with two 37.1, NF = 1 with four (spills) 45.8; at
-    // Norb = 12 (gradient in G, NA = 200): NF = 1 with three CTAs 3.8 ms, with two 4.2.
-    static constexpr int CTAS = NP <= 4 ? 4 : NP == 6 || NP == 10 || NP == 12 ? 3 : 2;
+    // Norb = 12 (gradient in G, NA = 200): NF = 1 with three CTAs 3.8 ms, with two 4.2. Norb = 8 (NA = 256, NE = 256, Nkz = 5):
+    // NF = 1 with four CTAs 1.79 ms, NF = 2 with two 1.84, NF = 1 with three 1.90; Norb = 6: NF = 2 0.90, NF = 1 0.97.
+    static constexpr int CTAS = NP <= 4 || NP == 8 ? 4 : NP <= 12 ? 3 : 2;
     static constexpr int XS = NP * NP * 2;          // floats of X per frequency
     static constexpr int US = 3 * NP * NP * 2;      // floats of U per frequency
     static constexpr int RSTR = (NP + 1) * 4;       // floats per column pair of the right operand (odd: bank spread)
@@ -269,6 +270,7 @@ __global__ void __launch_bounds__(128, TileShape<NP>::CTAS) spec_prod32_kernel(T
                     for (int dl = 0; dl < 2; ++dl)
 #pragma unroll
                         for (int j = 0; j < 3; ++j) {
+                            if (l + dl >= N) continue;  // the padding column of an odd block
                             const float4 b = lds4(R + j * CP * S::RSTR + (l + dl) * 4);
                             const float2 br = lo2(b), bi = hi2(b), nbi = f2neg(b.z, b.w);
 #pragma unroll
@@ -331,6 +333,7 @@ __global__ void __launch_bounds__(128, TileShape<NP>::CTAS) spec_prod32_kernel(T
                         for (int dm = 0; dm < 2; ++dm)
 #pragma unroll
                             for (int f = 0; f < NF; ++f) {
+                                if (m + dm >= N) continue;
                                 const float4 u = lds4(U + (size_t)f * c.fg * S::US + (i * NP + m + dm) * CP * 4);
                                 const float2 ur = lo2(u), ui = hi2(u), nui = f2neg(u.z, u.w);
 #pragma unroll

@@ -748,8 +748,8 @@ bool spectral_prod_tc_supported(const sse_dims& d) {
 
 // The tensor cores pay for large blocks with several bonds only: a tile of 128 rows costs about the same for every Norb
 // (the work around its GEMMs is a chain of latencies), and it holds fewer frequencies of few bonds. Products of both types,
-// tensor cores / FP32 CUDA cores, NA = 256, NE = 256, Nkz = 5: NB = 4: Norb 4 1169 / 393 us, 6 1783 / 897, 7 2280 / 2027, 8
-// 2361 / 1841, 9 3210 / 3704, 10 3275 / 3395; NB = 3: 8 1805 / 1395, 9 2501 / 2795, 10 2534 / 2561; NB = 1: 9 1071 / 989,
+// tensor cores / FP32 CUDA cores, NA = 256, NE = 256, Nkz = 5: NB = 4: Norb 4 1169 / 393 us, 6 1783 / 897, 7 2280 / 1780, 8
+// 2361 / 1795, 9 3210 / 3478, 10 3275 / 3395; NB = 3: 8 1805 / 1395, 9 2501 / 2620, 10 2534 / 2561; NB = 1: 9 1071 / 989,
 // 10 1067 / 900. The FP32 products keep more bits than the split FP16 operands.
 bool spectral_prod_tc_pays(const sse_dims& d) { return d.Norb >= 9 && d.NB >= 3; }
 
