@@ -135,7 +135,10 @@ struct RegDft {
     }
 };
 
-constexpr int kE4Cols = 8;  // columns per CTA: 128-byte rows of FP64 input, 64-byte rows of FP32
+// Columns per CTA: rows of 128 bytes, 8 columns of FP64 input or 16 of an FP32 spectrum (FinFET, inverse transform of S^,
+// both types: 8 columns 3.84 ms, 16 columns 3.18, 4 columns 5.41; G with 4 columns 6.42, with 8 4.70). The large codelets
+// keep 8, since two CTAs of 16 do not fit an SM.
+constexpr int kE4Cols = 8, kE4ColsWide = 16;
 
 // codelet lengths: the small set keeps two 24-point columns' worth of registers free for occupancy, the large one reaches
 // L = 36^2
@@ -169,12 +172,12 @@ __device__ __forceinline__ void e4_with(int n, F&& f) {
 
 struct E4Plan {
     int L, L1, L2, LP;  // L = L1 * L2; blocks of L2 rows padded to LP, an odd count (banks)
-    int threads, smem;  // one thread per column and codelet; tile + twiddle table
+    int cols, threads, smem;  // one thread per column and codelet; tile + twiddle table
     bool ok, large;
 };
 
 // the most balanced factorisation into two codelet lengths
-inline E4Plan make_e4_plan(int L) {
+inline E4Plan make_e4_plan(int L, bool wide) {
     E4Plan p{};
     p.L = L;
     for (int a = 4; a * a <= L; ++a)
@@ -182,27 +185,27 @@ inline E4Plan make_e4_plan(int L) {
     if (!p.ok) return p;
     p.LP = p.L2 | 1;
     p.large = p.L2 > kE4Small;
-    p.threads = (kE4Cols * p.L2 + 31) / 32 * 32;
-    p.smem = p.L1 * p.LP * kE4Cols * 8 + L * 8;
+    p.cols = wide && !p.large ? kE4ColsWide : kE4Cols;
+    p.threads = (p.cols * p.L2 + 31) / 32 * 32;
+    p.smem = p.L1 * p.LP * p.cols * 8 + L * 8;
     return p;
 }
 
-// CTA: kE4Cols adjacent columns of one batch (blockIdx.y). ld(batch, r, col) gives row r < L (zero where the loader
+// CTA: CC adjacent columns of one batch (blockIdx.y). ld(batch, r, col) gives row r < L (zero where the loader
 // pads), sv(batch, e, col, v) takes frequency rows e < sv.rows, as for fft_e_kernel. Pass 1 reads its rows from global
 // memory (all rows of a codelet in flight) and pass 2 writes its frequencies there: the tile crosses shared memory once,
 // with one barrier. The codelet lengths are run-time
 // choices inside one kernel, so every L = 2^a 3^b with two factors among them (all from 36 to 576 but a few) is served.
-// FinFET, two types: inverse transform of S^ 4.64 -> 3.84 ms (four barriers and the tile crossing shared memory four times
+// FinFET, two types: inverse transform of S^ 4.64 -> 3.18 ms (8 columns, four barriers and the tile crossing shared memory four times
 // before); L = 324 (NA = 90, Norb = 7): 97 -> 74 us against the Stockham kernel.
-template <int MOST>
-struct E4Bounds {  // at most 192 threads with four CTAs per SM (85 registers), or 288 with two (112)
-    static constexpr int THREADS = (kE4Cols * MOST + 31) / 32 * 32, CTAS = MOST <= kE4Small ? 4 : 2;
+template <int MOST, int CC>
+struct E4Bounds {  // 192 threads with four CTAs per SM or 384 with two (85 registers), 288 with two (112)
+    static constexpr int THREADS = (CC * MOST + 31) / 32 * 32, CTAS = MOST <= kE4Small && CC == kE4Cols ? 4 : 2;
 };
 
-template <int MOST, class Load, class Store>
-__global__ void __launch_bounds__(E4Bounds<MOST>::THREADS, E4Bounds<MOST>::CTAS)
+template <int MOST, int CC, class Load, class Store>
+__global__ void __launch_bounds__(E4Bounds<MOST, CC>::THREADS, E4Bounds<MOST, CC>::CTAS)
     fft_e4_kernel(E4Plan p, const float2* __restrict__ tw_g, Load ld, Store sv, size_t ncols) {
-    constexpr int CC = kE4Cols;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2* X = reinterpret_cast<float2*>(smem_raw);  // [L1][LP][CC]
     float2* tw = X + p.L1 * p.LP * CC;               // [L] exp(-2 pi i m / L)
@@ -241,13 +244,13 @@ __global__ void __launch_bounds__(E4Bounds<MOST>::THREADS, E4Bounds<MOST>::CTAS)
     });
 }
 
-template <int MOST, class Load, class Store>
+template <int MOST, int CC, class Load, class Store>
 cudaError_t launch_e4_t(const char* name, const E4Plan& p, const float2* tw, Load ld, Store sv, size_t ncols, int batches,
                         cudaStream_t st) {
-    auto kern = fft_e4_kernel<MOST, Load, Store>;
+    auto kern = fft_e4_kernel<MOST, CC, Load, Store>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p.smem);
     if (e != cudaSuccess) return e;
-    const size_t gx = (ncols + kE4Cols - 1) / kE4Cols;
+    const size_t gx = (ncols + CC - 1) / CC;
     if (gx == 0 || batches == 0) return cudaSuccess;
     if (gx > 0x7fffffffu || batches > 65535) return cudaErrorInvalidValue;
     SSE_TIMED(name, st, kern<<<dim3((unsigned)gx, (unsigned)batches), p.threads, p.smem, st>>>(p, tw, ld, sv, ncols));
@@ -305,7 +308,7 @@ size_t e4p_smem(const E4Plan& p, const Load& ld) {
 }
 
 template <int MOST, class Load, class Store>
-__global__ void __launch_bounds__(E4Bounds<MOST>::THREADS, MOST <= kE4Small ? 3 : 2)
+__global__ void __launch_bounds__(E4Bounds<MOST, kE4Cols>::THREADS, MOST <= kE4Small ? 3 : 2)
     fft_e4p_kernel(E4Plan p, const float2* __restrict__ tw_g, Load ld, Store sv, size_t ncols, int gx, int ntiles) {
     using Raw = typename Load::Raw;
     constexpr int CC = kE4Cols;
@@ -386,6 +389,10 @@ cudaError_t launch_e4p_t(const char* name, const E4Plan& p, const float2* tw, Lo
     return cudaGetLastError();
 }
 
+// loaders of an FP32 spectrum
+template <class Load>
+constexpr bool e4_wide = HasRawSrc<Load>::value && sizeof(typename HasRawSrcType<Load>::type) == 8;
+
 // The prefetching kernel for FP64 input tiles where the staging buffer fits: FinFET, transform of G, both types 4.70 ms
 // against 6.22 with fft_e4_kernel (the conversions hold up its loads); fft_e4_kernel for FP32 input, which needs none.
 template <int MOST, class Load, class Store>
@@ -395,7 +402,10 @@ cudaError_t launch_e4_any(const char* name, const E4Plan& p, const float2* tw, L
         if (e4p_smem(p, ld) <= (size_t)kE4pSmemMax)
             return launch_e4p_t<MOST>(e4_label(name, true), p, tw, ld, sv, ncols, batches, st);
     }
-    return launch_e4_t<MOST>(e4_label(name, false), p, tw, ld, sv, ncols, batches, st);
+    if constexpr (e4_wide<Load> && MOST <= kE4Small)
+        return launch_e4_t<MOST, kE4ColsWide>(e4_label(name, false), p, tw, ld, sv, ncols, batches, st);
+    else
+        return launch_e4_t<MOST, kE4Cols>(e4_label(name, false), p, tw, ld, sv, ncols, batches, st);
 }
 
 // FP32 E-transforms of the lengths with two codelet factors; every other length, and the FP64 transforms, take
@@ -404,7 +414,7 @@ template <class Load, class Store>
 cudaError_t launch_fft32(const char* name, const FftPlan& p, const typename Load::C* tw, Load ld, Store sv, size_t ncols,
                          int batches, cudaStream_t st) {
     if constexpr (std::is_same<typename Load::C, float2>::value) {
-        const E4Plan e4 = make_e4_plan(p.L);
+        const E4Plan e4 = make_e4_plan(p.L, e4_wide<Load>);
         if (e4.ok)
             return e4.large ? launch_e4_any<kE4Large>(name, e4, tw, ld, sv, ncols, batches, st)
                             : launch_e4_any<kE4Small>(name, e4, tw, ld, sv, ncols, batches, st);
