@@ -192,10 +192,10 @@ def mixed_useful_flops(d, mode: str) -> float:
 NCU_TRAFFIC = {
     "spec_prod_kernel": (4815.4, "a19635f8b1e45065", "atom-frequency of one type"),
     "spec_pi_kernel": (5033.6, "9a225dfc2cb7d028", "type-atom-frequency"),
-    "spec_adj_kernel": (13897.1, "3cadf5d36e3c5bb6", "atom-frequency of one type"),
-    "spec_prod32_kernel": (1923.2, "f34fb6e78487019a", "atom-frequency of one type"),
-    "spec_adj32_kernel": (7533.4, "8e9f1b2f0231170c", "atom-frequency of one type"),
-    "spec_pi32_kernel": (2121.4, "3f8eabc933beac4b", "type-atom-frequency"),
+    "spec_adj_kernel": (13895.7, "21baacdc342c7e76", "atom-frequency of one type"),
+    "spec_prod32_kernel": (1864.6, "3286cbe527227985", "atom-frequency of one type"),
+    "spec_adj32_kernel": (2735.9, "49aed8677f74242e", "atom-frequency of one type"),
+    "spec_pi32_kernel": (1982.9, "8f5da9c4210eb68b", "type-atom-frequency"),
     "spec_prod_tc_kernel": (1865.6, "b6487e717de45e49", "atom-frequency of one type"),
 }
 
