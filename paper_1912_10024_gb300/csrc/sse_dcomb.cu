@@ -8,8 +8,8 @@
 // rows: consecutive threads read and write consecutive 16-byte words, the neighbour lookup (dependent loads) and the
 // index arithmetic are paid once per thread, and sixteen independent loads are in flight per step.
 // What bounds them is not only HBM: six (forward) and four (adjoint) FP64 additions per complex entry take 163 and 108 us
-// on the FP64 pipe at the FinFET workload, against 87 us for the bytes of each. Measured there: forward 206 us, adjoint
-// 152 us (one thread per 144-byte block, nine strided words each: 214 and 279 us; one short-lived thread per entry and
+// on the FP64 pipe at the FinFET workload, against 87 us for the bytes of each. Measured there: forward 204 us, adjoint
+// 144 us (one thread per 144-byte block, nine strided words each: 214 and 279 us; one short-lived thread per entry and
 // four rows, which repeats the lookups: about 600 us each).
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -131,10 +131,11 @@ dcomb_bwd_kernel(sse_dims d, const int32_t* __restrict__ nbr, const double2* __r
     }
 }
 
-// cols threads across, and as many blocks down the `steps` row steps as fill the SMs a few times
+// cols threads across, and as many blocks down the `steps` row steps as make eight per SM, rounded down: the adjoint's 1188
+// blocks at FinFET are four full waves of two per SM (144 us), 1224 begin a fifth (152 us)
 dim3 dcomb_grid(size_t cols, int steps) {
     const size_t gx = (cols + kDcombThreads - 1) / kDcombThreads;
-    size_t gy = ((size_t)152 * 8 + gx - 1) / gx;
+    size_t gy = gx < 152 * 8 ? (size_t)152 * 8 / gx : 1;
     gy = gy < (size_t)steps ? gy : (size_t)steps;
     return dim3((unsigned)gx, (unsigned)(gy < 65535 ? gy : 65535));
 }
