@@ -128,7 +128,7 @@ __global__ void spec_prod_kernel(ProdCfg c, sse_dims d, FreqMap fm, const int32_
     }
 }
 
-// (S - S^H)/2 on the blocks of atoms in range. A CTA takes about 1024 elements of whole blocks through shared memory, so
+// (S - S^H)/2 on the blocks of atoms in range, where the inverse kz DFT does not project (Nkz > 8). A CTA takes about 1024 elements of whole blocks through shared memory, so
 // that the accesses are contiguous although every element meets its transposed one, and divides 64-bit indices once per
 // block. NA = 90, Norb = 7, NE = 301, Nkz = 4, both types: 131 -> 96 us (340 MB, 50 us; the FP64 operations 35 us). Forming
 // each pair of elements once halves those but adds a pass over shared memory: 120 us.
@@ -262,6 +262,10 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
     const TriMap tri = make_tri_map(d.Norb);
     const bool use_tri = half && tri_applies(d, L, (size_t)d.Nkz * L * scols);
     const size_t tg = (size_t)d.NA * tri.nt, ts = nA * tri.nt;  // columns
+    // symmetrised Sigma of general inputs: projected in the inverse kz DFT, then likewise by its triangle
+    const bool sym = (p.flags & SSE_FLAG_SYMMETRIZE) != 0;
+    const bool use_project = sym && !half && tri_applies(d, L, (size_t)-1);
+    const bool s_tri = use_tri || use_project;
     // the same for the 3 x 3 blocks of the lag kernel, whose triangle comes before that of G^ in S^'s region
     const TriMap tri3 = make_tri_map(3);
     const size_t tk = nA * d.NB * tri3.nt;
@@ -331,18 +335,18 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
         // 4. inverse transforms into Sigma^t
-        e = use_tri ? launch_kz_compress("dft_kz_compress_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st)
-                    : launch_dft_k("dft_kz_kernel(S)", Sh, d.Nkz, d.Nkz, (size_t)L * scols, 1, st);
+        e = use_tri       ? launch_kz_compress("dft_kz_compress_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st)
+            : use_project ? launch_kz_project("dft_kz_project_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st)
+                          : launch_dft_k("dft_kz_kernel(S)", Sh, d.Nkz, d.Nkz, (size_t)L * scols, 1, st);
         if (e != cudaSuccess) return e;
-        const double inv = 1.0 / ((double)d.Nkz * (double)L);
-        const bool sym = (p.flags & SSE_FLAG_SYMMETRIZE) != 0;
+        const double inv = (use_project ? 0.5 : 1.0) / ((double)d.Nkz * (double)L);
         // with `pipe` slice by slice, each handed to its download as soon as it is written
         const int sslices = pipe ? d.Nkz : 1, sper = pipe ? 1 : d.Nkz;
         sse_dims dk = d;
         dk.Nkz = sper;
         for (int k = 0; k < sslices; ++k) {
             double2* Sk = S[t] + (size_t)k * d.NE * d.NA * nel;
-            if (use_tri)
+            if (s_tri)
                 e = launch_fft32("fft_e_kernel(S)", plan, tw, LoadSpecConjT<C>{Sc + (size_t)k * L * ts, L, ts},
                                  StoreSigmaTri<C>{Sk, d.NE, gcols, (size_t)d.a_begin * nel, inv, d.NE, sym ? 1 : 0, tri},
                                  ts, sper, st);
@@ -350,7 +354,7 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
                 e = launch_fft32("fft_e_kernel(S)", plan, tw, LoadSpecConjT<C>{Sh + (size_t)k * L * scols, L, scols},
                                  StoreSigmaT<C>{Sk, d.NE, gcols, (size_t)d.a_begin * nel, inv, d.NE}, scols, sper, st);
             if (e != cudaSuccess) return e;
-            if (sym && !use_tri) {
+            if (sym && !s_tri) {
                 SSE_TIMED("symmetrize_kernel", st,
                           symmetrize_kernel<<<symmetrize_grid(d, sper), kSymThreads, 0, st>>>(dk, Sk));
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;

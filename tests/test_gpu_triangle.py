@@ -1,4 +1,4 @@
-"""SSE_FLAG_ANTIHERMITIAN: the transforms of the upper triangle's columns (sse_tri.cuh) against the general path of the
+"""Transforms of the upper triangle's columns (sse_tri.cuh), with SSE_FLAG_ANTIHERMITIAN against the general path of the
 same mode on the same anti-Hermitian inputs.
 
 kz grids with and without an instantiation (Nkz = 9 takes the full columns), odd and even transform lengths (self-paired
@@ -48,3 +48,21 @@ def test_pi_equals_general_path(d, mode, bound):
         R = B.pi(g.G_less, g.G_greater, g.dH, g.nbr, d.Nqz, d.Nw, **kw)
         for p, r in zip(P, R):
             assert normwise(p.cpu().numpy(), r.cpu().numpy()) <= bound
+
+
+@pytest.mark.parametrize("mode,bound", [("fp64_fft", 1e-12), ("fp32_fft", 2e-6), ("f16x3_fft", 2e-6)])
+@pytest.mark.parametrize("d", SHAPES, ids=lambda d: f"Norb{d.Norb}_NE{d.NE}_Nkz{d.Nkz}_NA{d.NA}")
+def test_projection_of_general_inputs(d, mode, bound):
+    """SSE_FLAG_SYMMETRIZE on inputs without symmetry: (S - S^H) / 2 of the unflagged result, exactly anti-Hermitian."""
+    if mode == "f16x3_fft" and d.Norb > 10:
+        pytest.skip("the tensor-core products take Norb <= 10")
+    g = make_inputs(d, seed=7, nbr=ring_neighbours(d.NA, d.NB), general=True).to("cuda")
+    args = (g.G_less, g.G_greater, g.dH, g.D_less, g.D_greater, g.nbr)
+    for atoms in ((0, d.NA), (2, 3)):
+        S = B.sigma(*args, mode=mode, symmetrize=True, atoms=atoms)
+        R = B.sigma(*args, mode=mode, atoms=atoms)
+        for s, r in zip(S, R):
+            s, r = s[:, :, atoms[0]:atoms[1]], r[:, :, atoms[0]:atoms[1]]
+            want = 0.5 * (r - r.conj().transpose(-1, -2))
+            assert normwise(s.cpu().numpy(), want.cpu().numpy()) <= bound
+            assert torch.equal(s, -s.conj().transpose(-1, -2))
