@@ -176,12 +176,14 @@ struct E4Plan {
     bool ok, large;
 };
 
-// the most balanced factorisation into two codelet lengths
+// the most balanced factorisation into two codelet lengths, the larger at most twice the smaller (in the pass of the shorter
+// DFTs a CTA's threads are idle in the ratio of the two: L = 243 = 9 * 27 lost, S^ 711 -> 939 us at NA = 1024, Norb = 6)
 inline E4Plan make_e4_plan(int L, bool wide) {
     E4Plan p{};
     p.L = L;
     for (int a = 4; a * a <= L; ++a)
-        if (L % a == 0 && e4_codelet(a, kE4Large) && e4_codelet(L / a, kE4Large)) p.L1 = a, p.L2 = L / a, p.ok = true;
+        if (L % a == 0 && L / a <= 2 * a && e4_codelet(a, kE4Large) && e4_codelet(L / a, kE4Large))
+            p.L1 = a, p.L2 = L / a, p.ok = true;
     if (!p.ok) return p;
     p.LP = p.L2 | 1;
     p.large = p.L2 > kE4Small;
@@ -196,7 +198,7 @@ inline E4Plan make_e4_plan(int L, bool wide) {
 // memory (all rows of a codelet in flight) and pass 2 writes its frequencies there: the tile crosses shared memory once,
 // with one barrier. The codelet lengths are run-time
 // choices inside one kernel, so every L = 2^a 3^b with two factors among them (all from 36 to 576 but a few) is served.
-// FinFET, two types: inverse transform of S^ 4.64 -> 3.18 ms (8 columns, four barriers and the tile crossing shared memory four times
+// FinFET, two types: inverse transform of S^ 4.64 -> 3.18 ms (8 columns, four barriers and four passes over shared memory
 // before); L = 324 (NA = 90, Norb = 7): 97 -> 74 us against the Stockham kernel.
 template <int MOST, int CC>
 struct E4Bounds {  // 192 threads with four CTAs per SM or 384 with two (85 registers), 288 with two (112)
@@ -408,6 +410,17 @@ cudaError_t launch_e4_any(const char* name, const E4Plan& p, const float2* tw, L
         return launch_e4_t<MOST, kE4Cols>(e4_label(name, false), p, tw, ld, sv, ncols, batches, st);
 }
 
+// FP64 tiles that are read in full but do not fit the staging buffer: the 27-point codelets (radix 3 only) lose to the
+// Stockham kernel there (G at NA = 512, Norb = 6: L = 729 1687 against 1290 us, L = 972 1760 against 1557; the 32 x 36
+// codelets of L = 1152 do not).
+template <class Load>
+bool e4_loses(const E4Plan& p, const Load& ld) {
+    if constexpr (HasRawSrc<Load>::value && sizeof(typename HasRawSrcType<Load>::type) == 16)
+        return (p.L1 == 27 || p.L2 == 27) && e4p_smem(p, ld) > (size_t)kE4pSmemMax;
+    else
+        return false;
+}
+
 // FP32 E-transforms of the lengths with two codelet factors; every other length, and the FP64 transforms, take
 // fft_e_kernel.
 template <class Load, class Store>
@@ -415,7 +428,7 @@ cudaError_t launch_fft32(const char* name, const FftPlan& p, const typename Load
                          int batches, cudaStream_t st) {
     if constexpr (std::is_same<typename Load::C, float2>::value) {
         const E4Plan e4 = make_e4_plan(p.L, e4_wide<Load>);
-        if (e4.ok)
+        if (e4.ok && !e4_loses(e4, ld))
             return e4.large ? launch_e4_any<kE4Large>(name, e4, tw, ld, sv, ncols, batches, st)
                             : launch_e4_any<kE4Small>(name, e4, tw, ld, sv, ncols, batches, st);
     }
