@@ -870,8 +870,8 @@ def main():
             roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None, "kernel": "sigma_fp64_fwd_kernel",
                     "peak_source": "derived: 152 SM x 2 DFMA/clk x 2 flop x 2070 MHz (DFMA probe: 1.25)"}
-        elif args.mode == "fp32_fft":
-            ks, n = kernel_s("spec_prod32_kernel")
+        elif args.mode == "fp32_fft" or (args.mode == "f16x3_fft" and "spec_prod_tc_kernel" not in kernels):
+            ks, n = kernel_s("spec_prod32_kernel")  # f16x3_fft: block sizes whose products run in FP32
             achieved = spectral_prod32_flops(d, args.antihermitian) / ks / 1e12
             roof = {"bound": "alu", "achieved": achieved, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
                     "frac": achieved / FP32_PEAK_TFLOPS,

@@ -390,8 +390,8 @@ cudaError_t launch_adj32_t(const Adj32Args& p, cudaStream_t st) {
     auto kern = spec_adj32_kernel<NP, ODD>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, AdjShape<NP>::smem);
     if (e != cudaSuccess) return e;
-    SSE_TIMED("spec_adj_kernel", st,
-              kern<<<dim3((unsigned)nA, (unsigned)c.nchunks, (unsigned)((p.d.NB + c.spc - 1) / c.spc)), AdjShape<NP>::THREADS, AdjShape<NP>::smem, st>>>(c, p));
+    const dim3 grid((unsigned)nA, (unsigned)c.nchunks, (unsigned)((p.d.NB + c.spc - 1) / c.spc));
+    SSE_TIMED("spec_adj_kernel", st, kern<<<grid, AdjShape<NP>::THREADS, AdjShape<NP>::smem, st>>>(c, p));
     return cudaGetLastError();
 }
 

@@ -128,10 +128,11 @@ __global__ void spec_prod_kernel(ProdCfg c, sse_dims d, FreqMap fm, const int32_
     }
 }
 
-// (S - S^H)/2 on the blocks of atoms in range, where the inverse kz DFT does not project (Nkz > 8). A CTA takes about 1024 elements of whole blocks through shared memory, so
-// that the accesses are contiguous although every element meets its transposed one, and divides 64-bit indices once per
-// block. NA = 90, Norb = 7, NE = 301, Nkz = 4, both types: 131 -> 96 us (340 MB, 50 us; the FP64 operations 35 us). Forming
-// each pair of elements once halves those but adds a pass over shared memory: 120 us.
+// (S - S^H)/2 on the blocks of atoms in range, where the inverse kz DFT does not project (Nkz > 8). A CTA takes about 1024
+// elements of whole blocks through shared memory, so that the accesses are contiguous although every element meets its
+// transposed one, and divides 64-bit indices once per block. NA = 90, Norb = 7, NE = 301, Nkz = 4, both types: 131 -> 96 us
+// (340 MB, 50 us; the FP64 operations 35 us). Forming each pair of elements once halves those but adds a pass over shared
+// memory: 120 us.
 constexpr int kSymElems = 1024, kSymThreads = 256;
 
 __global__ void __launch_bounds__(kSymThreads) symmetrize_kernel(sse_dims d, double2* __restrict__ S) {
