@@ -128,11 +128,11 @@ __global__ void spec_prod_kernel(ProdCfg c, sse_dims d, FreqMap fm, const int32_
     }
 }
 
-// (S - S^H)/2 on the blocks of atoms in range, where the inverse kz DFT does not project (Nkz > 8). A CTA takes about 1024
-// elements of whole blocks through shared memory, so that the accesses are contiguous although every element meets its
-// transposed one, and divides 64-bit indices once per block. NA = 90, Norb = 7, NE = 301, Nkz = 4, both types: 131 -> 96 us
-// (340 MB, 50 us; the FP64 operations 35 us). Forming each pair of elements once halves those but adds a pass over shared
-// memory: 120 us.
+// (S - S^H)/2 on the blocks of atoms in range: FP32 spectra, and FP64 ones where the inverse kz DFT does not project
+// (Nkz > 8). A CTA takes about 1024 elements of whole blocks through shared memory, so that the accesses are contiguous
+// although every element meets its transposed one, and divides 64-bit indices once per block. NA = 90, Norb = 7, NE = 301,
+// Nkz = 4, both types: 131 -> 96 us (340 MB, 50 us; the FP64 operations 35 us). Forming each pair of elements once halves
+// those but adds a pass over shared memory: 120 us.
 constexpr int kSymElems = 1024, kSymThreads = 256;
 
 __global__ void __launch_bounds__(kSymThreads) symmetrize_kernel(sse_dims d, double2* __restrict__ S) {
@@ -263,10 +263,12 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
     const TriMap tri = make_tri_map(d.Norb);
     const bool use_tri = half && tri_applies(d, L, (size_t)d.Nkz * L * scols);
     const size_t tg = (size_t)d.NA * tri.nt, ts = nA * tri.nt;  // columns
-    // symmetrised Sigma of general inputs: projected in the inverse kz DFT, then likewise by its triangle
+    // Symmetrised Sigma of general inputs: projected in the inverse kz DFT, then likewise by its triangle. FP64 spectra only:
+    // the symmetrisation is FP64 arithmetic in every mode, so FP32 spectra are transformed back in full and
+    // symmetrize_kernel averages each pair of elements, anti-Hermitian inputs included.
     const bool sym = (p.flags & SSE_FLAG_SYMMETRIZE) != 0;
-    const bool use_project = sym && !half && tri_applies(d, L, (size_t)-1);
-    const bool s_tri = use_tri || use_project;
+    const bool use_project = sizeof(T) == 8 && sym && !half && tri_applies(d, L, (size_t)-1);
+    const bool s_tri = use_project || (use_tri && (sizeof(T) == 8 || !sym));
     // the same for the 3 x 3 blocks of the lag kernel, whose triangle comes before that of G^ in S^'s region
     const TriMap tri3 = make_tri_map(3);
     const size_t tk = nA * d.NB * tri3.nt;
@@ -330,15 +332,20 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
                           pc, d, fm, p.nbr, p.dH, Gh, Kh, Sh, p.scale, status));
         }
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (half && !use_tri) {
+        if (half && !s_tri) {
             SSE_TIMED("mirror_sigma_kernel", st,
                       mirror_sigma_kernel<<<grid_for(fm.count * nA * nel, 256), 256, 0, st>>>(fm, nA, d.Norb, Sh));
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
         // 4. inverse transforms into Sigma^t
-        e = use_tri       ? launch_kz_compress("dft_kz_compress_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st)
-            : use_project ? launch_kz_project("dft_kz_project_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st)
-                          : launch_dft_k("dft_kz_kernel(S)", Sh, d.Nkz, d.Nkz, (size_t)L * scols, 1, st);
+        if (use_project) {
+            if constexpr (sizeof(T) == 8)
+                e = launch_kz_project("dft_kz_project_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st);
+        } else if (s_tri) {
+            e = launch_kz_compress("dft_kz_compress_kernel(S)", Sh, Sc, tri, d.Nkz, L, ts, st);
+        } else {
+            e = launch_dft_k("dft_kz_kernel(S)", Sh, d.Nkz, d.Nkz, (size_t)L * scols, 1, st);
+        }
         if (e != cudaSuccess) return e;
         const double inv = (use_project ? 0.5 : 1.0) / ((double)d.Nkz * (double)L);
         // with `pipe` slice by slice, each handed to its download as soon as it is written

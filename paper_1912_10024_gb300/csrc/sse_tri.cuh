@@ -158,10 +158,11 @@ __global__ void __launch_bounds__(256) dft_kz_compress_kernel(const C* __restric
     }
 }
 
-// Symmetrised Sigma of general inputs: the spectrum of (S - S^H) / 2 is (S^_mn(f) - conj(S^_nm(-f))) / 2, anti-Hermitian, so
-// its triangle is enough. Inverse kz DFT of twice that from the full blocks S[kappa][eps][atom][mn] into the triangle's
-// columns (the store halves it): the symmetrisation costs no pass of its own and 0.45 of the inverse E-transform goes away.
-// NA = 90, Norb = 7, NE = 301, Nkz = 4, FP32, both types: kz pass, inverse E-transform and symmetrisation 192 -> 118 us.
+// Symmetrised Sigma of general inputs, FP64 spectra: the spectrum of (S - S^H) / 2 is (S^_mn(f) - conj(S^_nm(-f))) / 2,
+// anti-Hermitian, so its triangle is enough. Inverse kz DFT of twice that from the full blocks S[kappa][eps][atom][mn] into
+// the triangle's columns (the store halves it): the symmetrisation costs no pass of its own and 0.45 of the inverse
+// E-transform goes away. Not for FP32 spectra: there the projection would round to 24 bits what symmetrize_kernel averages
+// in FP64.
 template <class C, int NK>
 __global__ void __launch_bounds__(256) dft_kz_project_kernel(const C* __restrict__ S, C* __restrict__ X, TriMap t, int L,
                                                              unsigned ncols) {
