@@ -104,6 +104,16 @@ struct Adj32Args {
     unsigned* status;
 };
 
+// s + x, with the rounding error of the addition, exact in FP32 (Knuth's TwoSum), added to e. The up to 64 group sums of a
+// flush keep the bits that FP64 additions would (an e of at most 64 errors of 2^-24 loses less than 2^-40), without the
+// narrow FP64 pipe's additions and conversions. Adjoint at the FinFET workload, both types: 109.6 ms, against 117.5 with
+// FP64 additions and 108.4 with rounded FP32 ones.
+__device__ __forceinline__ void two_sum(float& s, float& e, float x) {
+    const float t = s + x, b = t - s;
+    e += (s - (t - b)) + (x - b);
+    s = t;
+}
+
 template <int NP, int ODD>
 __global__ void __launch_bounds__(AdjShape<NP>::THREADS, AdjShape<NP>::CTAS) spec_adj32_kernel(Adj32Cfg c, Adj32Args p) {
     using S = AdjShape<NP>;
@@ -344,7 +354,7 @@ __global__ void __launch_bounds__(AdjShape<NP>::THREADS, AdjShape<NP>::CTAS) spe
                 }
             }
             if (++chain < S::FLUSH && tile + 1 < tile1) continue;
-            // flush: sum the groups (FP32, fixed order), add to this chunk's FP64 partial
+            // flush: sum the groups (fixed order) and add to this chunk's FP64 partial
             chain = 0;
             __syncthreads();  // phase 2 is done with X_mu and U_mu
             float2* sAcc = reinterpret_cast<float2*>(sX);  // [2 GP][3][nel]
@@ -365,10 +375,22 @@ __global__ void __launch_bounds__(AdjShape<NP>::THREADS, AdjShape<NP>::CTAS) spe
             const double inv = p.scale / (double)p.nfreq;
             double2* part_out = p.gdh_part + (((size_t)blockIdx.y * nA + la) * d.NB + s) * 3 * nel;
             for (int i = tid; i < 3 * nel; i += nt) {  // entry i belongs to one thread
-                float2 sum = make_float2(0.f, 0.f);
+                float2 sum = make_float2(0.f, 0.f), low = sum;
 #pragma unroll
-                for (int g = 0; g < 2 * S::GP; ++g) sum = cadd(sum, sAcc[g * 3 * nel + i]);
-                double2 v = make_double2((double)sum.x * inv, (double)sum.y * inv);
+                for (int g = 0; g < 2 * S::GP; ++g) {
+                    const float2 x = sAcc[g * 3 * nel + i];
+                    two_sum(sum.x, low.x, x.x);
+                    two_sum(sum.y, low.y, x.y);
+                }
+                double2 v = make_double2((double)sum.x + (double)low.x, (double)sum.y + (double)low.y);
+                if (!isfinite(sum.x) || !isfinite(sum.y)) {  // the sum or one of its terms leaves the FP32 range
+                    v = make_double2(0.0, 0.0);
+                    for (int g = 0; g < 2 * S::GP; ++g) {
+                        const float2 x = sAcc[g * 3 * nel + i];
+                        v = make_double2(v.x + (double)x.x, v.y + (double)x.y);
+                    }
+                }
+                v = make_double2(v.x * inv, v.y * inv);
                 if (!first) {
                     const double2 o = part_out[i];
                     v = make_double2(v.x + o.x, v.y + o.y);

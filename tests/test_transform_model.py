@@ -263,8 +263,9 @@ def test_fp32_arithmetic_error_is_within_the_stated_bound():
 
 
 def coupling_gradient_terms(nbr, dH, Dl, Dg, Gl, Wl, dt):
-    """Per-frequency terms of the coupling gradient of one type (the summand of grad dH_m above), in the complex
-    type dt: [bond][m][frequency][Norb][Norb]."""
+    """Terms of the coupling gradient of one type in the complex type dt, as spec_adj32_kernel adds them: per bond two
+    arrays [(frequency, l)][m][Norb][Norb], X_mu[:, l] conj(G[:, l]) with X_mu = sum_j -i conj(K_mu,j) W A_j, and
+    conj(W[l, :]) U_mu[l, :] with U_mu = sum_i i K_i,mu A_i G."""
     Nkz, NE, NA, Norb, _ = Gl.shape
     Nqz, Nw = Dl.shape[0], Dl.shape[1]
     NB = nbr.shape[1]
@@ -273,62 +274,72 @@ def coupling_gradient_terms(nbr, dH, Dl, Dg, Gl, Wl, dt):
     def spectrum(X):
         Xp = np.zeros((Nkz, L) + X.shape[2:], dt)
         Xp[:, :NE] = X
-        return np.fft.fft2(Xp, axes=(0, 1))
+        return np.fft.fft2(Xp, axes=(0, 1)).reshape((Nkz * L,) + X.shape[2:])
 
     Gh, Wh = spectrum(Gl), spectrum(Wl)
     K = np.zeros((Nkz, L, NA, NB, 3, 3), dt)
     for w in range(Nw):
         K[:Nqz, w + 1] = Dl[:, w]
         K[:Nqz, L - (w + 1)] = Dg[:, w]
-    Kh = np.fft.fft2(K, axes=(0, 1))
+    Kh = np.fft.fft2(K, axes=(0, 1)).reshape(Nkz * L, NA, NB, 3, 3)
     terms = []
     for a in range(NA):
         for s in range(NB):
-            A, Wa, Gb = dH[a, s].astype(dt), Wh[:, :, a], Gh[:, :, nbr[a, s]]
-            Q = [Wa @ A[j] @ np.conj(np.swapaxes(Gb, -1, -2)) for j in range(3)]
-            R = [np.conj(np.swapaxes(Wa, -1, -2)) @ A[i] @ Gb for i in range(3)]
-            terms.append([sum((-1j * np.conj(Kh[:, :, a, s, m, j]))[..., None, None] * Q[j]
-                              + (1j * Kh[:, :, a, s, j, m])[..., None, None] * R[j] for j in range(3))
-                          .reshape(Nkz * L, Norb, Norb) for m in range(3)])
+            A, W, G, k = dH[a, s].astype(dt), Wh[:, a], Gh[:, nbr[a, s]], Kh[:, a, s]
+            X = np.einsum("fmj,fjab->fmab", -1j * np.conj(k), np.stack([W @ A[j] for j in range(3)], 1)).astype(dt)
+            U = np.einsum("fim,fiab->fmab", 1j * k, np.stack([A[i] @ G for i in range(3)], 1)).astype(dt)
+            terms.append((np.einsum("fmxl,fyl->flmxy", X, np.conj(G)).reshape(-1, 3, Norb, Norb),
+                          np.einsum("flx,fmly->flmxy", np.conj(W), U).reshape(-1, 3, Norb, Norb)))
     return terms
 
 
-def lane_sums_fp32(x, chunk, lanes):
-    """The kernel's order: chunks of `chunk` frequencies; within a chunk lane f adds frequencies f, f + lanes, ...
-    one after another in FP32; lanes and chunks are then added in FP64."""
-    total = np.zeros(x.shape[1:], np.complex128)
-    for c0 in range(0, x.shape[0], chunk):
-        for f in range(lanes):
-            acc = np.zeros(x.shape[1:], np.complex64)
-            for v in x[c0 + f:min(x.shape[0], c0 + chunk):lanes]:
-                acc = (acc + v).astype(np.complex64)
-            total += acc
-    return total
+def group_sums_fp32(x, tile, tiles, groups):
+    """The kernel's order: group g of a tile of `tile` (frequency, l) terms adds the terms g, g + groups, ... in FP32, on
+    through `tiles` tiles; then the groups and the runs of `tiles` tiles are added in FP64."""
+    steps = (tile + groups - 1) // groups
+    pad = np.zeros((-(-x.shape[0] // (tile * tiles)) * tiles, steps * groups) + x.shape[1:], np.complex64)
+    for t in range(pad.shape[0]):
+        part = x[t * tile:(t + 1) * tile]
+        pad[t, :part.shape[0]] = part
+    pad = pad.reshape((-1, tiles * steps, groups) + x.shape[1:])
+    acc = np.zeros_like(pad[:, 0])
+    for i in range(pad.shape[1]):
+        acc = acc + pad[:, i]
+    assert acc.dtype == np.complex64
+    return acc.astype(np.complex128).sum((0, 1))
 
 
-def test_fp32_coupling_gradient_needs_short_lane_sums():
+@pytest.mark.parametrize("Norb,F,groups", [(2, 128, 32), (10, 10, 6), (16, 4, 4)])
+def test_fp32_coupling_gradient_needs_short_chains(Norb, F, groups):
     """On a FinFET-sized frequency grid (Nkz = 7, L = 576, 4032 frequencies) the coupling-gradient terms computed in
-    FP32 and added per lane in FP32 drift from the FP64 sums when a lane adds ~270 terms (the chunks of three per atom
-    at 1024 atoms, 5 lanes); chunks of at most 32 terms per lane, added in FP64, stay close to the floor set by the
-    FP32 terms themselves."""
+    FP32 and added per group of threads in FP32 drift from the FP64 sums when a chain runs through the frequencies of a
+    whole chunk (a third of them); chains of at most 192 additions (two per term, as in spec_adj32_kernel), added in
+    FP64, stay close to the floor set by the FP32 terms themselves. F and groups: the kernel's frequencies per tile and
+    groups per half of phase 2 at the block size. Bound of the short chains: n terms of random sign, each addition rounded
+    to 2^-24 of a partial sum that grows as the square root of its terms, leave 2^-24 sqrt(n / 2) of the sum beside the
+    floor."""
     from paper_1912_10024_gb300.inputs import make_upstream
-    d = Dims(NA=2, NB=2, Norb=10, NE=512, Nkz=7, Nqz=7, Nw=32)
+    d = Dims(NA=2, NB=1, Norb=Norb, NE=512, Nkz=7, Nqz=7, Nw=32)
     x = make_inputs(d, seed=41, nbr=ring_neighbours(d.NA, d.NB))
     W, _ = make_upstream(d, seed=42)
     arrs = [t.numpy() for t in (x.nbr, x.dH, x.D_less, x.D_greater, x.G_less)] + [W.numpy()]
-    ref = np.array([[t.sum(0) for t in b] for b in coupling_gradient_terms(*arrs, np.complex128)])
-    t32 = coupling_gradient_terms(*arrs, np.complex64)
-    nfreq = t32[0][0].shape[0]
-    lanes = 5
-
-    def err(sums):
-        return np.abs(np.array(sums) - ref).max() / np.abs(ref).max()
-
-    floor = err([[t.astype(np.complex128).sum(0) for t in b] for b in t32])
-    long_chunks = err([[lane_sums_fp32(t, nfreq // 3, lanes) for t in b] for b in t32])
-    short_chunks = err([[lane_sums_fp32(t, 32 * lanes, lanes) for t in b] for b in t32])
-    assert long_chunks > 2 * short_chunks, (floor, long_chunks, short_chunks)
-    assert short_chunks < 2 * floor, (floor, long_chunks, short_chunks)
+    tile = F * Norb
+    flush = 192 // (2 * -(-tile // groups))  # tiles between two flushes
+    third = 4032 // 3 // F
+    ref, floor, long_chains, short_chains = [], [], [], []
+    for p, q in zip(coupling_gradient_terms(*arrs, np.complex128), coupling_gradient_terms(*arrs, np.complex64)):
+        assert q[0].dtype == np.complex64
+        ref.append(sum(t.sum(0) for t in p))
+        floor.append(sum(t.astype(np.complex128).sum(0) for t in q))
+        long_chains.append(sum(group_sums_fp32(t, tile, third, groups) for t in q))
+        short_chains.append(sum(group_sums_fp32(t, tile, flush, groups) for t in q))
+    ref = np.array(ref)
+    floor, long_chains, short_chains = (np.abs(np.array(v) - ref).max() / np.abs(ref).max()
+                                        for v in (floor, long_chains, short_chains))
+    terms = -(-tile // groups) * flush  # per chain
+    if third > flush:  # (a chunk of blocks of 2 x 2 is shorter than a chain)
+        assert long_chains > 2 * short_chains, (floor, long_chains, short_chains)
+    assert short_chains < floor + 2.0 ** -24 * math.sqrt(terms / 2), (floor, long_chains, short_chains)
 
 
 def sigma_spectrum(nbr, dH, Dt, Dtb, G, Nw):
