@@ -5,10 +5,12 @@
 // the slot s' with nbr[b][s'] = a (symmetric neighbour lists). No atomics, so the results are deterministic.
 //
 // Both kernels are gathers. A thread keeps its column (the same for every (qz, w)) and walks down the
-// rows: consecutive threads read and write consecutive 16-byte words, the neighbour lookup (dependent loads) and the
-// index arithmetic are paid once per thread, and sixteen independent loads are in flight per step.
+// rows: consecutive threads read and write consecutive 16-byte words, and the neighbour lookup (dependent loads) and the
+// index arithmetic are paid once per thread. The forward takes a row at a time, eight independent loads, with four CTAs
+// per SM: with two rows and two CTAs it took the same 204 us at the FinFET workload, but 60 us instead of 34 for one row of
+// NA = 32000, NB = 4 (a thread per block: 40) and 131 instead of 78 for one row of NA = 16384, NB = 16.
 // What bounds them is not only HBM: six (forward) and four (adjoint) FP64 additions per complex entry take 163 and 108 us
-// on the FP64 pipe at the FinFET workload, against 87 us for the bytes of each. Measured there: forward 204 us, adjoint
+// on the FP64 pipe at the FinFET workload, against 87 us for the bytes of each. Measured there: forward 205 us, adjoint
 // 144 us (one thread per 144-byte block, nine strided words each: 214 and 279 us; one short-lived thread per entry and
 // four rows, which repeats the lookups: about 600 us each).
 #include <cuda_runtime.h>
@@ -29,8 +31,8 @@ constexpr int kDcombThreads = 256;
 constexpr int kDcombTableBonds = 64;  // bonds per atom up to which the adjoint keeps its reverse bonds in shared memory
 
 // Dc[q][w][a][s] for atoms in range; bonds without a reverse slot (or an out-of-range
-// neighbour) get zero and raise the status bit. One thread per output entry of a row, two rows at a time.
-__global__ void __launch_bounds__(kDcombThreads, 2)
+// neighbour) get zero and raise the status bit. One thread per output entry of a row, both types of a row at a time.
+__global__ void __launch_bounds__(kDcombThreads, 4)
 dcomb_fwd_kernel(sse_dims d, const int32_t* __restrict__ nbr, const double2* __restrict__ raw_l,
                  const double2* __restrict__ raw_g, double2* __restrict__ Dl, double2* __restrict__ Dg,
                  unsigned* __restrict__ status) {
@@ -49,17 +51,15 @@ dcomb_fwd_kernel(sse_dims d, const int32_t* __restrict__ nbr, const double2* __r
     const size_t o = a * bw + (size_t)bond * 9 + e;
     const int rows = d.Nqz * d.Nw;
     const size_t rp = d.NA * rw, op = d.NA * bw;  // row pitches
-    for (int r = blockIdx.y * 2; r < rows; r += gridDim.y * 2) {
-        const size_t r1 = r + 1 < rows ? r + 1 : r;  // an odd last row is formed twice
-        const double2 *l0 = raw_l + r * rp, *l1 = raw_l + r1 * rp, *g0 = raw_g + r * rp, *g1 = raw_g + r1 * rp;
-        const double2 x[4] = {l0[ba], g0[ba], l1[ba], g1[ba]}, y[4] = {l0[bb], g0[bb], l1[bb], g1[bb]};
-        const double2 z[4] = {l0[aa], g0[aa], l1[aa], g1[aa]}, u[4] = {l0[ab], g0[ab], l1[ab], g1[ab]};
+    for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+        const double2 *l = raw_l + r * rp, *g = raw_g + r * rp;
+        const double2 x[2] = {l[ba], g[ba]}, y[2] = {l[bb], g[bb]}, z[2] = {l[aa], g[aa]}, u[2] = {l[ab], g[ab]};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 2; ++k) {
             double2 v = make_double2(0.0, 0.0);
             if (ok)  // left to right
                 v = make_double2(x[k].x - y[k].x - z[k].x + u[k].x, x[k].y - y[k].y - z[k].y + u[k].y);
-            ((k & 1) ? Dg : Dl)[(k < 2 ? r : r1) * op + o] = v;
+            (k ? Dg : Dl)[r * op + o] = v;
         }
     }
 }
@@ -144,7 +144,7 @@ dim3 dcomb_grid(size_t cols, int steps) {
 
 cudaError_t dcomb_fwd(const sse_dims& d, const int32_t* nbr, const double2* raw_l, const double2* raw_g,
                       double2* Dl, double2* Dg, unsigned* status, cudaStream_t st) {
-    const dim3 grid = dcomb_grid((size_t)(d.a_end - d.a_begin) * d.NB * 9, (d.Nqz * d.Nw + 1) / 2);
+    const dim3 grid = dcomb_grid((size_t)(d.a_end - d.a_begin) * d.NB * 9, d.Nqz * d.Nw);
     SSE_TIMED("dcomb_fwd_kernel", st,
               dcomb_fwd_kernel<<<grid, kDcombThreads, 0, st>>>(d, nbr, raw_l, raw_g, Dl, Dg, status));
     return cudaGetLastError();

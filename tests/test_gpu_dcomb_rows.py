@@ -1,6 +1,7 @@
-"""The bond-weight kernels at the edges of their work split: (qz, w) row counts around the four rows of a thread, column
-counts around a block, one to four bonds, and lists in which some bonds have no reverse (zero weight, zero gradient,
-status reported). The reference adds the same terms in numpy in the order of Eq. (3): the forward is equal to the bit,
+"""The bond-weight kernels at the edges of their work split: few (qz, w) rows, column counts around a block, so many
+columns that a thread walks down several rows, one to eight bonds around the four of an adjoint step, more bonds than the
+adjoint's table of reverse bonds holds, and lists in which some bonds have no reverse (zero weight, zero gradient, status
+reported). The reference adds the same terms in numpy in the order of Eq. (3): the forward is equal to the bit,
 and so is the adjoint (slot sums of two terms, self blocks subtracted bond by bond)."""
 import numpy as np
 import pytest
@@ -24,6 +25,9 @@ def reverse_slots(nbr):
 @pytest.mark.parametrize("NA,NB,Nqz,Nw,steps", [
     (3, 1, 1, 1, [1]), (2, 1, 1, 3, [1]), (13, 2, 2, 2, [1, -1]), (15, 2, 5, 1, [1, -1]), (7, 4, 3, 3, [1, -1, 2, -2]),
     (12, 3, 2, 4, [1, -1, 3]), (33, 3, 1, 7, [2, -2, 5]),
+    (17, 5, 1, 3, [1, -1, 2, -2, 4]), (19, 7, 2, 2, [1, -1, 2, -2, 3, -3, 5]), (20, 8, 1, 5, [1, -1, 2, -2, 3, -3, 4, -4]),
+    (66, 65, 1, 3, [s for k in range(1, 33) for s in (k, -k)] + [33]),
+    (3000, 2, 1, 13, [1, -1]),  # 211 and 106 blocks across: 5 and 11 of the 13 rows at once
 ], ids=str)
 def test_row_and_column_remainders(NA, NB, Nqz, Nw, steps):
     nbr = np.array([[(a + s) % NA for s in steps] for a in range(NA)], dtype=np.int32)
