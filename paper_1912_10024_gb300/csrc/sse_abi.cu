@@ -47,7 +47,7 @@ bool op_supported(const sse_dims& d, int mode, Op op) {
         case Op::Fwd:
             if (mode == SSE_MODE_TF32 || mode == SSE_MODE_BF16X3) return sse::mixed_supported(d, mode);
             if (mode == SSE_MODE_F16X3_FFT) return sse::spectral_fwd_tc_supported(d);
-            return mode == SSE_MODE_FP64 || sse::spectral_fwd_supported(d, fp32);
+            return mode == SSE_MODE_FP64 || sse::spectral_fwd_supported(d);
         case Op::Bwd: return mode == SSE_MODE_FP64 || sse::spectral_bwd_supported(d);
         case Op::BwdG: return sse::spectral_bwd_g_supported(d, fp32);  // transforms in every mode it takes
         case Op::Pi: return sse::spectral_pi_supported(d);              // limits of the FP64 and FP32 kernels

@@ -259,19 +259,19 @@ cudaError_t launch_e4_t(const char* name, const E4Plan& p, const float2* tw, Loa
     return cudaGetLastError();
 }
 
-// profile labels of the register-codelet kernels (plain, prefetching) for a transform the drivers name
-// "fft_e_kernel(X)"
+// profile labels of the register-codelet kernels (plain, and prefetching for the FP64 inputs that it takes) for a transform
+// the drivers name "fft_e_kernel(X)"
 inline const char* e4_label(const char* name, bool prefetch) {
     static const char* const labels[][3] = {
         {"fft_e_kernel(G)", "fft_e4_kernel(G)", "fft_e4p_kernel(G)"},
-        {"fft_e_kernel(K)", "fft_e4_kernel(K)", "fft_e4p_kernel(K)"},
-        {"fft_e_kernel(S)", "fft_e4_kernel(S)", "fft_e4p_kernel(S)"},
         {"fft_e_kernel(W)", "fft_e4_kernel(W)", "fft_e4p_kernel(W)"},
-        {"fft_e_kernel(H)", "fft_e4_kernel(H)", "fft_e4p_kernel(H)"},
-        {"fft_e_kernel(R)", "fft_e4_kernel(R)", "fft_e4p_kernel(R)"},
-        {"fft_e_kernel(C)", "fft_e4_kernel(C)", "fft_e4p_kernel(C)"}};
+        {"fft_e_kernel(K)", "fft_e4_kernel(K)"},
+        {"fft_e_kernel(S)", "fft_e4_kernel(S)"},
+        {"fft_e_kernel(H)", "fft_e4_kernel(H)"},
+        {"fft_e_kernel(R)", "fft_e4_kernel(R)"},
+        {"fft_e_kernel(C)", "fft_e4_kernel(C)"}};
     for (const auto& l : labels)
-        if (strcmp(l[0], name) == 0) return l[prefetch ? 2 : 1];
+        if (strcmp(l[0], name) == 0 && l[prefetch ? 2 : 1]) return l[prefetch ? 2 : 1];
     return name;
 }
 

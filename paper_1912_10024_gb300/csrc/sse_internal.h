@@ -93,7 +93,7 @@ int spectral_length(const sse_dims& d);
 bool spectral_supported(const sse_dims& d);
 // The forward's limits for FP64 (fp32 = false) or FP32 (true) transforms and block products; like every
 // *_supported predicate below, a host-only function of the sizes that the entry points test before any device work.
-bool spectral_fwd_supported(const sse_dims& d, bool fp32);
+bool spectral_fwd_supported(const sse_dims& d);
 size_t spectral_fwd_workspace(const sse_dims& d);
 cudaError_t spectral_fwd(const Problem& p, double2* S_less, double2* S_greater, unsigned* status, void* ws,
                          size_t ws_bytes, cudaStream_t st);

@@ -45,11 +45,7 @@ __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); 
 
 template <int B>
 __device__ __forceinline__ void tile_cp_async(float* dst, const void* src, bool ok) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    if constexpr (B == 16)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(ok ? 16 : 0) : "memory");
-    else
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(ok ? 8 : 0) : "memory");
+    cp_async_elem<B>((uint32_t)__cvta_generic_to_shared(dst), src, ok);
 }
 __device__ __forceinline__ void tile_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void tile_cp_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }

@@ -95,28 +95,8 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-// 8-byte shared-memory access of two consecutive floats
+// 8-byte shared-memory load of two consecutive floats
 __device__ __forceinline__ float2 ld2(const float* p) { return *reinterpret_cast<const float2*>(p); }
-__device__ __forceinline__ void st2(float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); }
-
-// acc[dm][dn] (re/im in ar/ai, index dm * 2 + dn) += x[dm] * y[dn], x or y conjugated on request: 16 FMAs
-template <bool CONJX, bool CONJY>
-__device__ __forceinline__ void cmac2x2(float* ar, float* ai, float2 xr, float2 xi, float2 yr, float2 yi) {
-    const float sx = CONJX ? -1.f : 1.f, sy = CONJY ? -1.f : 1.f;
-    const float xrv[2] = {xr.x, xr.y}, xiv[2] = {sx * xi.x, sx * xi.y};
-    const float yrv[2] = {yr.x, yr.y}, yiv[2] = {sy * yi.x, sy * yi.y};
-#pragma unroll
-    for (int dm = 0; dm < 2; ++dm)
-#pragma unroll
-        for (int dn = 0; dn < 2; ++dn) {
-            const int q = dm * 2 + dn;
-            ar[q] = fmaf(xrv[dm], yrv[dn], ar[q]);
-            ar[q] = fmaf(-xiv[dm], yiv[dn], ar[q]);
-            ai[q] = fmaf(xrv[dm], yiv[dn], ai[q]);
-            ai[q] = fmaf(xiv[dm], yrv[dn], ai[q]);
-        }
-}
-
 
 // complex element type of the transforms: double2 (FP64 modes) or float2 (FP32_FFT)
 template <class C>
@@ -294,7 +274,6 @@ struct LoadGT {
     __device__ const Raw* src(int k, int r, size_t col) const { return G + ((size_t)k * NE + r) * ncols + col; }
     static __device__ C cvt(Raw v) { return CT<C>::mk(v.x, v.y); }
 };
-using LoadG = LoadGT<double2>;
 // lag kernel of one qz slice: row w+1 <- D^t(q,w), row L-(w+1) <- D^t'(q,w), else zero.
 // col over (a - a_begin, s, ij); D rows have NA*NB*9 entries, the range starts at a_begin*NB*9.
 template <class CC>
@@ -312,7 +291,6 @@ struct LoadLagT {
         return CT<C>::mk(v.x, v.y);
     }
 };
-using LoadLag = LoadLagT<double2>;
 // spectrum [k][eps][col], conjugated (inverse transform = conj(FFT(conj(x))))
 template <class CC>
 struct LoadSpecConjT {
@@ -326,7 +304,6 @@ struct LoadSpecConjT {
     __device__ const Raw* src(int k, int r, size_t col) const { return X + ((size_t)k * L + r) * ncols + col; }
     static __device__ C cvt(Raw v) { return cconj(v); }
 };
-using LoadSpecConj = LoadSpecConjT<double2>;
 
 template <class C>
 struct StoreSpecT {  // out[batch][r][col]
@@ -336,7 +313,6 @@ struct StoreSpecT {  // out[batch][r][col]
     int rows;
     __device__ void operator()(int b, int r, size_t col, C v) const { X[((size_t)b * L + r) * ncols + col] = v; }
 };
-using StoreSpec = StoreSpecT<double2>;
 template <class C>
 struct StoreSigmaT {  // S[k][E][a_begin*nel + col] = conj(v) * inv in FP64, E < NE
     double2* S;
@@ -350,7 +326,6 @@ struct StoreSigmaT {  // S[k][E][a_begin*nel + col] = conj(v) * inv in FP64, E <
         S[((size_t)k * NE + r) * rowlen + col0 + col] = make_double2((double)(v.x * s), (double)(-v.y * s));
     }
 };
-using StoreSigma = StoreSigmaT<double2>;
 
 template <class Load, class Store, int CC>
 __global__ void __launch_bounds__(kFftThreads) fft_e_kernel(FftPlan p,
@@ -557,10 +532,6 @@ __device__ __forceinline__ void put3(T* P, int nel, int e, C v) {
     P[nel + e] = v.y;
     P[2 * nel + e] = v.x + v.y;
 }
-
-// The FP32 tile kernels place the tile threads of two adjacent frequencies in one warp; per-frequency strides of
-// 16 mod 32 floats put their rows of a plane on disjoint shared-memory banks.
-inline int bank_pad16(int floats) { return floats + ((16 - floats % 32) + 32) % 32; }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 

@@ -265,19 +265,17 @@ __global__ void spec_gdh_reduce_kernel(sse_dims d, int nchunks, const double2* _
     }
 }
 
-// upstream gradient gS^t[k][E][a][mn] of atoms in range, optionally projected to (W - W^H)/2
+// upstream gradient gS^t[k][E][a][mn] of atoms in range, projected to (W - W^H)/2
 template <class CC>
 struct LoadWT {
     using C = CC;
     const double2* W;
     int NE, Norb;
     size_t rowlen, col0;
-    int sym;
     __device__ C operator()(int k, int r, size_t col) const {
         if (r >= NE) return CT<C>::mk(0, 0);
         const double2* row = W + ((size_t)k * NE + r) * rowlen + col0;
         const double2 x = row[col];
-        if (!sym) return CT<C>::mk(x.x, x.y);
         const int nel = Norb * Norb;
         const size_t blk = col / nel;
         const int mn = (int)(col - blk * nel), mm = mn / Norb, nn = mn - mm * Norb;
@@ -285,7 +283,6 @@ struct LoadWT {
         return CT<C>::mk(0.5 * (x.x - y.x), 0.5 * (x.y + y.y));
     }
 };
-using LoadW = LoadWT<double2>;
 
 // E-transform of the upstream gradient into W^ [k][eps][nA * nel]; without the projection its elements are plain reads,
 // which the prefetching transform of G takes (FinFET, both types: 6.3 -> 4.7 ms)
@@ -296,7 +293,7 @@ cudaError_t launch_fft_w(const FftPlan& plan, const C* tw, const double2* W, con
     const size_t cols = (size_t)(d.a_end - d.a_begin) * nel;
     const StoreSpecT<C> out{Wh, L, cols, L};
     if (!sym) return launch_fft32("fft_e_kernel(W)", plan, tw, LoadGT<C>{W + col0, d.NE, rowlen}, out, cols, d.Nkz, st);
-    return launch_fft32("fft_e_kernel(W)", plan, tw, LoadWT<C>{W, d.NE, d.Norb, rowlen, col0, sym}, out, cols, d.Nkz, st);
+    return launch_fft32("fft_e_kernel(W)", plan, tw, LoadWT<C>{W, d.NE, d.Norb, rowlen, col0}, out, cols, d.Nkz, st);
 }
 
 // grad D^t (rows l = w+1) and grad D^t' (rows L-(w+1)) from the inverse transform of H^t:

@@ -204,10 +204,7 @@ bool spectral_supported(const sse_dims& d) {
 }
 
 // The FP32 product kernel takes every block size and bond count of spectral_supported.
-bool spectral_fwd_supported(const sse_dims& d, bool fp32) {
-    (void)fp32;
-    return spectral_supported(d);
-}
+bool spectral_fwd_supported(const sse_dims& d) { return spectral_supported(d); }
 
 size_t spectral_fwd_workspace(const sse_dims& d) { return spec_layout(d).total; }
 size_t spectral_fwd32_workspace(const sse_dims& d) { return spec_layout(d, 8).total; }
@@ -225,7 +222,7 @@ cudaError_t spectral_fwd_t(const Problem& p, double2* S_less, double2* S_greater
     const sse_dims& d = p.d;
     // tc: mode F16X3_FFT, the FP32 transforms with the block products on the tensor cores where those are faster
     if (tc && sizeof(T) != 4) return cudaErrorNotSupported;
-    if (!(tc ? spectral_fwd_tc_supported(d) : spectral_fwd_supported(d, sizeof(T) == 4))) return cudaErrorNotSupported;
+    if (!(tc ? spectral_fwd_tc_supported(d) : spectral_fwd_supported(d))) return cudaErrorNotSupported;
     const SpecLayout lay = spec_layout(d, sizeof(C));
     if (ws_bytes < lay.total) return cudaErrorInvalidValue;
     unsigned char* base = static_cast<unsigned char*>(ws);
@@ -391,7 +388,7 @@ cudaError_t spectral_fwd32(const Problem& p, double2* S_less, double2* S_greater
 }
 
 bool spectral_fwd_tc_supported(const sse_dims& d) {
-    return spectral_fwd_supported(d, true) && spectral_prod_tc_supported(d);
+    return spectral_fwd_supported(d) && spectral_prod_tc_supported(d);
 }
 
 cudaError_t spectral_fwd_tc(const Problem& p, double2* S_less, double2* S_greater, unsigned* status, void* ws,

@@ -465,7 +465,6 @@ struct StorePiT {
             make_double2(-(double)v.y * inv_scale, -(double)v.x * inv_scale);
     }
 };
-using StorePi = StorePiT<double2>;
 
 // (P - P^H)/2 on every 3x3 block of the atoms in range
 __global__ void symmetrize3_kernel(sse_dims d, double2* __restrict__ P) {

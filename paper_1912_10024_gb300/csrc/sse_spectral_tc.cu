@@ -704,6 +704,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 template <int NORB>
 cudaError_t launch_tc(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, const double2* dH, const float2* Gh,
                       const float2* Kh, float2* Sh, double scale, unsigned* status, cudaStream_t st) {
+    static_assert(2 * TcShape<NORB>::TM_P + kTcMaxNB * TcShape<NORB>::TM_O <= 512, "TMEM columns");
     const TcCfg c = make_tc_cfg<NORB>(d, fm.count);
     if (c.nitems == 0) return cudaSuccess;
     static int nsm = 0;
@@ -722,29 +723,10 @@ cudaError_t launch_tc(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, 
     return cudaGetLastError();
 }
 
-template <int NORB>
-bool tc_fits(const sse_dims& d) {
-    const TcCfg c = make_tc_cfg<NORB>(d, 1);
-    return d.NB <= kTcMaxNB && c.smem <= 227 * 1024 && 2 * TcShape<NORB>::TM_P + d.NB * TcShape<NORB>::TM_O <= 512;
-}
-
 }  // namespace
 
-bool spectral_prod_tc_supported(const sse_dims& d) {
-    switch (d.Norb) {
-        case 1: return tc_fits<1>(d);
-        case 2: return tc_fits<2>(d);
-        case 3: return tc_fits<3>(d);
-        case 4: return tc_fits<4>(d);
-        case 5: return tc_fits<5>(d);
-        case 6: return tc_fits<6>(d);
-        case 7: return tc_fits<7>(d);
-        case 8: return tc_fits<8>(d);
-        case 9: return tc_fits<9>(d);
-        case 10: return tc_fits<10>(d);
-        default: return false;
-    }
-}
+// the mode's limits, those of its tensor-core kernel
+bool spectral_prod_tc_supported(const sse_dims& d) { return d.Norb <= 10 && d.NB <= kTcMaxNB; }
 
 // The tensor cores pay for large blocks with several bonds only: a tile of 128 rows costs about the same for every Norb
 // (the work around its GEMMs is a chain of latencies), and it holds fewer frequencies of few bonds. Products of both types,
