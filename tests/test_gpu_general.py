@@ -7,7 +7,8 @@ every result is compared element by element with the FP64 oracle, which takes G 
 Bounds (normwise max|gpu - oracle| / max|oracle| per output tensor), the same as each mode's own tests:
 FP64 and FP64_FFT 1e-12; FP32_FFT 2e-6 (forward, Pi), 1e-5 (adjoint, G-gradient); F16X3_FFT 2e-6; BF16X3 2e-5;
 TF32 2e-3.
-Shapes: the tiny workload, and Norb = 10 with ragged energy tiles and Nqz < Nkz.
+Shapes: the tiny workload, and Norb = 10 with ragged energy tiles and Nqz < Nkz, with two bonds and with four (F16X3_FFT
+takes the tensor cores for three bonds and more at this block size).
 """
 import math
 
@@ -23,7 +24,8 @@ from paper_1912_10024_gb300.inputs import TINY, Dims, make_inputs, make_upstream
 pytestmark = pytest.mark.gpu
 SCALE = 1.0 / (2.0 * math.pi)
 NORB10 = Dims(NA=5, NB=2, Norb=10, NE=40, Nkz=3, Nqz=2, Nw=11)
-SHAPES = [TINY, NORB10]
+FOUR_BONDS = Dims(NA=6, NB=4, Norb=10, NE=37, Nkz=3, Nqz=2, Nw=7)
+SHAPES = [TINY, NORB10, FOUR_BONDS]
 FWD_BOUND = {"fp64": 1e-12, "fp64_fft": 1e-12, "fp32_fft": 2e-6, "f16x3_fft": 2e-6, "bf16x3": 2e-5, "tf32": 2e-3}
 BWD_BOUND = {"fp64": 1e-12, "fp64_fft": 1e-12, "fp32_fft": 1e-5}
 
@@ -53,9 +55,10 @@ def test_forward(dims, mode):
     assert max(errs) <= FWD_BOUND[mode], errs
 
 
+@pytest.mark.parametrize("dims", [NORB10, FOUR_BONDS], ids=_ids)
 @pytest.mark.parametrize("mode", ["fp64_fft", "fp32_fft", "f16x3_fft"])
-def test_host_buffer_forward(mode):
-    inp = _general(NORB10, seed=1100)
+def test_host_buffer_forward(mode, dims):
+    inp = _general(dims, seed=1100)
     pin = [t.pin_memory() for t in (inp.G_less, inp.G_greater, inp.dH, inp.D_less, inp.D_greater, inp.nbr)]
     S = B.sigma_host(*pin, mode=mode, check=True)
     O = oracle.sigma(inp.nbr, inp.dH, inp.D_less, inp.D_greater, inp.G_less, inp.G_greater, SCALE)

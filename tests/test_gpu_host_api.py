@@ -1,9 +1,13 @@
 """Host-buffer forward (sse_sigma_fwd_host): uploads, compute and downloads on two streams, G and Sigma handed over
 one kz slice at a time, give the same bytes as the device-pointer entry point, for every kind of mode and with the
 symmetrisation and anti-Hermitian flags, and write only the rows of the atom range."""
+import math
+
 import pytest
 import torch
 
+import oracle
+from conftest import normwise
 from paper_1912_10024_gb300 import binding as B
 from paper_1912_10024_gb300.inputs import TINY, Dims, make_inputs, ring_neighbours
 
@@ -48,15 +52,24 @@ def test_one_stream_is_refused():
     assert e.value.status == 1
 
 
-@pytest.mark.parametrize("mode", ["fp64_fft", "fp32_fft"])
+@pytest.mark.parametrize("d", [Dims(NA=7, NB=2, Norb=3, NE=50, Nkz=9, Nqz=4, Nw=7),
+                               Dims(NA=6, NB=3, Norb=5, NE=33, Nkz=3, Nqz=2, Nw=3),
+                               Dims(NA=5, NB=4, Norb=10, NE=29, Nkz=8, Nqz=8, Nw=3),
+                               Dims(NA=5, NB=2, Norb=4, NE=20, Nkz=1, Nqz=1, Nw=4)], ids=lambda d: f"Nkz{d.Nkz}")
+@pytest.mark.parametrize("mode", ["fp64_fft", "fp32_fft", "f16x3_fft"])
 @pytest.mark.parametrize("flags", [("symmetrize",), ("antihermitian",), ("symmetrize", "antihermitian")])
-def test_flags_same_bytes_many_slices(mode, flags):
-    """Nkz = 9 kz slices: the per-slice transforms, symmetrisation and downloads match the device call bit for bit."""
-    d = Dims(NA=7, NB=2, Norb=3, NE=50, Nkz=9, Nqz=4, Nw=7)
-    inp = make_inputs(d, seed=64, nbr=ring_neighbours(7, 2))
+def test_flags_same_bytes_many_slices(mode, flags, d):
+    """The per-slice transforms, symmetrisation and downloads match the device call bit for bit, and the oracle: with
+    Nkz = 9 kz slices of full columns, and with up to eight slices whose transforms take triangles (FP64_FFT: the projection
+    too; Norb = 10 with four bonds: F16X3_FFT on the tensor cores)."""
+    inp = make_inputs(d, seed=64, nbr=ring_neighbours(d.NA, d.NB), general=flags == ("symmetrize",))
     Gl, Gg, dH, Dl, Dg, nbr = host_inputs(inp, True)
     kw = {f: True for f in flags}
-    Hl, Hg = B.sigma_host(Gl, Gg, dH, Dl, Dg, nbr, mode=mode, check=True, **kw)
+    H = B.sigma_host(Gl, Gg, dH, Dl, Dg, nbr, mode=mode, check=True, **kw)
     g = inp.to("cuda")
-    Sl, Sg = B.sigma(g.G_less, g.G_greater, g.dH, g.D_less, g.D_greater, g.nbr, mode=mode, check=True, **kw)
-    assert torch.equal(Hl, Sl.cpu()) and torch.equal(Hg, Sg.cpu())
+    S = B.sigma(g.G_less, g.G_greater, g.dH, g.D_less, g.D_greater, g.nbr, mode=mode, check=True, **kw)
+    O = oracle.sigma(inp.nbr, inp.dH, inp.D_less, inp.D_greater, inp.G_less, inp.G_greater, 1.0 / (2.0 * math.pi))
+    for h, s, o in zip(H, S, O):
+        assert torch.equal(h, s.cpu())
+        o = 0.5 * (o - o.conj().swapaxes(-1, -2)) if "symmetrize" in flags else o
+        assert normwise(h.numpy(), o) <= (1e-12 if mode == "fp64_fft" else 2e-6)
