@@ -228,6 +228,12 @@ def ncu_traffic(kernel: str, units: float):
     return per * units
 
 
+def compare_steps(mode: str, warmup: int, steps: int):
+    """Warm-up and timed steps of another mode on the run's inputs: the run's own, but one and at most two for the direct
+    FP64 kernel, a minute per step at the default workload (twenty of them would take most of half an hour)."""
+    return (1, min(steps, 2)) if mode == "fp64" else (max(3, warmup), steps)
+
+
 def gpu_local_cpus(dev):
     """Host CPUs on the GPU's own NUMA node (sysfs local_cpulist of its PCI device), intersected with the CPUs this
     process may use; None when the system does not say."""
@@ -660,21 +666,21 @@ def main():
                 if rc != 0:
                     raise B.SseError(rc, "sse_sigma_fwd")
 
-            mw = 1 if mname == "fp64" else max(3, args.warmup)  # the direct FP64 kernel runs about a minute
+            mw, ms = compare_steps(mname, args.warmup, args.steps)
             for _ in range(mw):
                 mstep()
             torch.cuda.synchronize(dev)
             m0, m1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             m0.record(stream)
-            for _ in range(args.steps):
+            for _ in range(ms):
                 mstep()
             m1.record(stream)
             torch.cuda.synchronize(dev)
-            mms = m0.elapsed_time(m1) / args.steps
+            mms = m0.elapsed_time(m1) / ms
             err = max(float((Ml - ref[0]).abs().max() / ref[0].abs().max()),
                       float((Mg - ref[1]).abs().max() / ref[1].abs().max()))
             compare[mname] = {"value": uf / (mms * 1e-3) / 1e12, "unit": "TFLOP/s", "ms_per_step": mms,
-                              "warmup": mw, "speedup_of_this_run": mms / ms_per_step,
+                              "warmup": mw, "steps": ms, "speedup_of_this_run": mms / ms_per_step,
                               "max_normwise_diff_vs_this_run": err, "stated_bound_vs_oracle": bounds[mname]}
             del wsm, Ml, Mg
         del ref

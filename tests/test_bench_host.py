@@ -161,3 +161,10 @@ def test_clock_samples_come_from_the_gpu_torch_uses(monkeypatch):
     clk.lines = ["1965, 2070, 900.1, Not Active, Not Active, Not Active, Active", "garbage"]
     out = clk.summary()
     assert out == {"sm_mhz": 1965.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"], "samples": 1, "gpu": "7"}
+
+
+def test_direct_fp64_comparison_is_bounded():
+    """The comparison with the direct FP64 kernel, a minute per step at the default workload, does not grow with --steps;
+    the other modes take the run's own step counts."""
+    assert bench.compare_steps("fp64", 5, 20) == (1, 2) and bench.compare_steps("fp64", 3, 1) == (1, 1)
+    assert bench.compare_steps("f16x3_fft", 5, 20) == (5, 20) and bench.compare_steps("tf32", 1, 4) == (3, 4)
