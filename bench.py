@@ -194,7 +194,7 @@ NCU_TRAFFIC = {
     "spec_pi_kernel": (5033.6, "9a225dfc2cb7d028", "type-atom-frequency"),
     "spec_adj_kernel": (13895.7, "21baacdc342c7e76", "atom-frequency of one type"),
     "spec_prod32_kernel": (1864.6, "3286cbe527227985", "atom-frequency of one type"),
-    "spec_adj32_kernel": (2735.9, "49aed8677f74242e", "atom-frequency of one type"),
+    "spec_adj32_kernel": (2722.8, "3a8ffead054cde59", "atom-frequency of one type"),
     "spec_pi32_kernel": (1982.9, "8f5da9c4210eb68b", "type-atom-frequency"),
     "spec_prod_tc_kernel": (1865.6, "b6487e717de45e49", "atom-frequency of one type"),
 }

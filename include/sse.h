@@ -127,10 +127,11 @@ typedef enum sse_mode {
  *             sse_profile_read reports the device time per kernel.
  * ANTIHERMITIAN : the caller states that every Norb x Norb block of G^< and G^>
  *             (and, for sse_sigma_fwd, every 3x3 block of D^< and D^>) is exactly
- *             anti-Hermitian, as lesser and greater Green's functions are. The
- *             FP64_FFT forward and sse_pi_fwd then compute one frequency of each
- *             pair (f, -f) and obtain the other from Sigma^(-f) = -Sigma^(f)^H,
- *             C^(-f) = C^(f)^H (half the block products). With CHECK the inputs are
+ *             anti-Hermitian, as lesser and greater Green's functions are. The forward
+ *             in FP64_FFT, FP32_FFT and F16X3_FFT and sse_pi_fwd then compute one
+ *             frequency of each pair (f, -f) and obtain the other from
+ *             Sigma^(-f) = -Sigma^(f)^H, C^(-f) = C^(f)^H (half the block products), and
+ *             read the blocks' upper triangles only where that is enough. With CHECK the inputs are
  *             verified bit for bit and a violation is reported as
  *             SSE_ERR_DEVICE_CHECK; without it the results for inputs that are not
  *             anti-Hermitian are unspecified. Ignored by the other modes and entries. */

@@ -14,9 +14,9 @@
 // (frequency, l) in GP: 5.5 FMAs per float loaded. W^, G^ and K^ of the next tile arrive by cp.async meanwhile, so a tile
 // takes two barriers. FMAs are issued in pairs along the dimension in which the shared operand is stored in pairs, so
 // that only the other operand has to be duplicated in registers.
-// FinFET: 99.3 -> 91.5 ms for both types (0.53 of the FP32 pipe in useful work; ncu at the adjoint workload: FMA pipe 62%
-// active, shared-memory wavefronts 60%, two warps per scheduler waiting on fixed latencies); NF = 1 with three CTAs per SM
-// 92.7 ms, with four (spills) 99.9.
+// FinFET: 99.3 -> 92.8 ms for both types (0.52 of the FP32 pipe in useful work; ncu at the adjoint workload: FMA pipe 61%
+// active, shared-memory wavefronts 58%, two warps per scheduler waiting on fixed latencies). Measured with the groups' sums
+// rounded: NF = 2 with two CTAs per SM 91.5 ms, NF = 1 with three 92.7, with four (spills) 99.9.
 #pragma once
 
 #include "sse_prod32.cuh"
@@ -24,7 +24,7 @@
 namespace sse {
 namespace {
 
-// The sums of phase 2 are flushed to FP64 after at most this many FP32 additions into one of them: the chain of the
+// The sums of phase 2 are flushed to the FP64 partial after at most this many FP32 additions into one of them: the chain of the
 // previous kernel (32 frequencies of six terms per lane). Without the flush a chunk of 320 frequencies put the coupling
 // gradient at the FinFET workload 7.7e-7 from the 64-bit value instead of 4.7e-7.
 constexpr int kAdj32ChainTerms = 192;

@@ -7,10 +7,10 @@
 // Both kernels are gathers. A thread keeps its column (the same for every (qz, w)) and walks down the
 // rows: consecutive threads read and write consecutive 16-byte words, and the neighbour lookup (dependent loads) and the
 // index arithmetic are paid once per thread. The forward takes a row at a time, eight independent loads, with four CTAs
-// per SM: with two rows and two CTAs it took the same 204 us at the FinFET workload, but 60 us instead of 34 for one row of
+// per SM: with two rows and two CTAs it took 204 us at the FinFET workload, but 60 us instead of 34 for one row of
 // NA = 32000, NB = 4 (a thread per block: 40) and 131 instead of 78 for one row of NA = 16384, NB = 16.
 // What bounds them is not only HBM: six (forward) and four (adjoint) FP64 additions per complex entry take 163 and 108 us
-// on the FP64 pipe at the FinFET workload, against 87 us for the bytes of each. Measured there: forward 205 us, adjoint
+// on the FP64 pipe at the FinFET workload, against 87 us for the bytes of each. Measured there: forward 207 us, adjoint
 // 144 us (one thread per 144-byte block, nine strided words each: 214 and 279 us; one short-lived thread per entry and
 // four rows, which repeats the lookups: about 600 us each).
 #include <cuda_runtime.h>

@@ -412,7 +412,8 @@ cudaError_t launch_e4_any(const char* name, const E4Plan& p, const float2* tw, L
 
 // FP64 tiles that are read in full but do not fit the staging buffer: the 27-point codelets (radix 3 only) lose to the
 // Stockham kernel there (G at NA = 512, Norb = 6: L = 729 1687 against 1290 us, L = 972 1760 against 1557; the 32 x 36
-// codelets of L = 1152 do not).
+// codelets of L = 1152 do not). The pairs without 27 of two such lengths lose as well: 18 x 36 of L = 648 557 against 515 us,
+// 24 x 36 of L = 864 729 against 576 (the same sizes, Nkz = 2).
 template <class Load>
 bool e4_loses(const E4Plan& p, const Load& ld) {
     if constexpr (HasRawSrc<Load>::value && sizeof(typename HasRawSrcType<Load>::type) == 16)

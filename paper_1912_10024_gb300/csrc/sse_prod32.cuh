@@ -6,13 +6,12 @@
 // with X = G^_b, T_j = dH_j, k = K^ for the forward, and X = W^_a, T_j = dH_j^H, k = conj(K^) over the incoming bonds
 // for the gradient in G: one kernel serves both.
 //
-// What bounds it: the FP32 pipe (128 FMA per clock and SM, 80 TFLOP/s) and, next to it, the shared-memory return path
-// (128 bytes per clock and SM, also for a broadcast: a 16-byte load by a warp takes 4 clocks, the issue time of 16
-// warp-wide FMAs). A thread therefore owns half of the rows and two columns of the block, for the three j together and
-// for NF frequencies: at Np = 10 P takes 7.5 FMAs and acc 4.4 per float loaded, against 2 on 2 x 2 tiles for the P_j one
+// What bounds it: the shared-memory return path (128 bytes per clock and SM, also for a broadcast: a 16-byte load by a warp
+// takes 4 clocks, the issue time of 16 warp-wide FMAs) and, next to it, the FP32 pipe (128 FMA per clock and SM, 80
+// TFLOP/s). A thread therefore owns half of the rows and two columns of the block, for the three j together and for NF
+// frequencies: at Np = 10 (NF = 1) P takes 5.5 FMAs and acc 2.9 per float loaded, against 2 on 2 x 2 tiles for the P_j one
 // frequency at a time. FinFET workload, per step of two types: 52.3 -> 36.6 ms (0.62 of the FP32 pipe; ncu at the
-// adjoint workload: FMA pipe 62% active with the inner loops rolled, shared-memory wavefronts 47%, two warps per
-// scheduler waiting on fixed latencies).
+// adjoint workload: shared-memory wavefronts 72% of peak, FMA pipe 69% active, three warps per scheduler).
 #pragma once
 
 #include "sse_spectral.cuh"
@@ -71,8 +70,8 @@ struct TileShape {
     static constexpr int CP = NP / 2;               // column pairs
     static constexpr int TPF = 2 * CP;              // threads per frequency set
     static constexpr int NF = NP <= 6 ? 2 : 1;      // frequencies per thread: two while their tiles fit in registers
-    // CTAs per SM that the registers (P 12 Np NF / 2, acc 2 Np NF, operands) leave room for without spills. Measured at
-    // Norb = 10: NF = 1 with three CTAs 36.6 ms per FinFET step, NF = 2 with two 37.1, NF = 1 with four (spills) 45.8; at
+    // CTAs per SM that the registers (P 12 Np NF / 2, acc 2 Np NF, operands) leave room for with at most 16 bytes of spills
+    // (Np = 4, 6, 8 and 12; none at 10). Measured at Norb = 10: NF = 1 with three CTAs 36.6 ms per FinFET step, NF = 2 with two 37.1, NF = 1 with four (spills) 45.8; at
     // Norb = 12 (gradient in G, NA = 200): NF = 1 with three CTAs 3.8 ms, with two 4.2. Norb = 8 (NA = 256, NE = 256, Nkz = 5):
     // NF = 1 with four CTAs 1.79 ms, NF = 2 with two 1.84, NF = 1 with three 1.90; Norb = 6: NF = 2 0.90, NF = 1 0.97.
     static constexpr int CTAS = NP <= 4 || NP == 8 ? 4 : NP <= 12 ? 3 : 2;

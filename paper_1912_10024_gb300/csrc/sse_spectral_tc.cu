@@ -729,10 +729,13 @@ cudaError_t launch_tc(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, 
 bool spectral_prod_tc_supported(const sse_dims& d) { return d.Norb <= 10 && d.NB <= kTcMaxNB; }
 
 // The tensor cores pay for large blocks with several bonds only: a tile of 128 rows costs about the same for every Norb
-// (the work around its GEMMs is a chain of latencies), and it holds fewer frequencies of few bonds. Products of both types,
-// tensor cores / FP32 CUDA cores, NA = 256, NE = 256, Nkz = 5: NB = 4: Norb 4 1169 / 393 us, 6 1783 / 897, 7 2280 / 1780, 8
-// 2361 / 1795, 9 3210 / 3478, 10 3275 / 3395; NB = 3: 8 1805 / 1395, 9 2501 / 2620, 10 2534 / 2561; NB = 1: 9 1071 / 989,
-// 10 1067 / 900. The FP32 products keep more bits than the split FP16 operands.
+// (the work around its GEMMs is a chain of latencies), and the work per item and tile is shared by the bonds. Products of
+// both types, tensor cores / FP32 CUDA cores, NA = 256, NE = 256, Nkz = 5: NB = 4: Norb 4 1169 / 393 us, 6 1783 / 897, 7 2280 /
+// 1780, 8 2361 / 1795, 9 3212 / 3483, 10 3278 / 3404; NB = 3: 8 1805 / 1395, 9 2499 / 2633, 10 2543 / 2568; NB = 2: 9 1802 /
+// 1788, 10 1829 / 1739; NB = 1: 9 1077 / 948, 10 1073 / 907. NA = 1024, NE = 512, Nkz = 3, Norb 9 and 10: NB = 4 15.01 / 16.17
+// ms, 15.38 / 15.79; 3 11.69 / 12.21, 11.88 / 11.92; 2 8.37 / 8.28, 8.47 / 8.05. NA = 90, NE = 301, Nkz = 4: NB = 4 1074 / 1144
+// us, 1095 / 1105; 3 837 / 869, 850 / 840 (the one reversal, by 1%); 2 610 / 610, 620 / 582. The FP32 products keep more bits
+// than the split FP16 operands.
 bool spectral_prod_tc_pays(const sse_dims& d) { return d.Norb >= 9 && d.NB >= 3; }
 
 cudaError_t spectral_prod_tc(const sse_dims& d, const FreqMap& fm, const int32_t* nbr, const double2* dH,

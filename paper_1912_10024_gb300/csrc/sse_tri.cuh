@@ -14,7 +14,9 @@ namespace sse {
 namespace {
 
 constexpr int kTriMaxNorb = 16, kTriMax = kTriMaxNorb * (kTriMaxNorb + 1) / 2;
-constexpr int kTriMaxNk = 8;  // kz grids with an instantiation of the kernels below (larger ones take the full columns)
+// kz grids with an instantiation of the kernels below: up to 8 the two FP64 columns of a thread leave registers for two CTAs
+// per SM (compress: 124 at Nkz = 8, 170 at 12, 230 at 16). Larger grids take the full columns; not measured there.
+constexpr int kTriMaxNk = 8;
 
 struct TriMap {  // the upper triangle of an n x n block, row by row
     int nt, nel;
@@ -161,7 +163,8 @@ __global__ void __launch_bounds__(256) dft_kz_compress_kernel(const C* __restric
 // Symmetrised Sigma of general inputs, FP64 spectra: the spectrum of (S - S^H) / 2 is (S^_mn(f) - conj(S^_nm(-f))) / 2,
 // anti-Hermitian, so its triangle is enough. Inverse kz DFT of twice that from the full blocks S[kappa][eps][atom][mn] into
 // the triangle's columns (the store halves it): the symmetrisation costs no pass of its own and 0.45 of the inverse
-// E-transform goes away. Not for FP32 spectra: there the projection would round to 24 bits what symmetrize_kernel averages
+// E-transform goes away. FP64_FFT, both types, kz pass, inverse E-transform and symmetrisation: NA = 90, Norb = 7, NE = 301,
+// Nkz = 4 993 -> 585 us, NA = 256, Norb = 10, NE = 256, Nkz = 5 6.01 -> 3.27 ms. Not for FP32 spectra: there the projection would round to 24 bits what symmetrize_kernel averages
 // in FP64.
 template <class C, int NK>
 __global__ void __launch_bounds__(256) dft_kz_project_kernel(const C* __restrict__ S, C* __restrict__ X, TriMap t, int L,
