@@ -3,8 +3,8 @@
 // of Sigma. So G is transformed along E for those columns only, the kz DFT that follows writes the full blocks of the
 // computed half of the frequencies (and of the other half where Pi needs it), and after the products the inverse kz DFT
 // reads that half and writes the triangle's columns for every frequency. 0.55 of the E-transforms at Norb = 10, half of
-// the kz passes, no mirror pass, no separate symmetrisation. The 3 x 3 blocks of the lag kernel are taken the same way (six
-// columns of nine). FinFET in FP64 (the transforms are bound by the FP64 pipe): E-transforms of G and S 102 -> 58 ms, of K
+// the kz passes, no mirror pass, no separate symmetrisation (symmetrised FP32 spectra excepted: mirrored, transformed back
+// in full and averaged in FP64). The 3 x 3 blocks of the lag kernel are taken the same way (six columns of nine). FinFET in FP64 (the transforms are bound by the FP64 pipe): E-transforms of G and S 102 -> 58 ms, of K
 // 17.6 -> 11.8; kz passes 36 -> 21 ms, mirror 3.6 -> 0: the call 830 -> 761 ms.
 #pragma once
 
